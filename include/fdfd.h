@@ -127,11 +127,9 @@ typedef struct {
                                   pivot rows, then to FP64, as above; the next design refactor then
                                   refactors the whole symmetric form again.  FP64 factors are
                                   always LU. */
-  int sweep_rhs_pairs;         /* 1: the sweeps of complex FP32 factors take the right-hand sides of a
-                                  wavelength two at a time when their count is even (each factor entry
-                                  loaded once for both; twice the shared memory per CTA); 0: one at a
-                                  time (default: the second system's reads mostly hit the caches, and
-                                  the pairs' shared memory lowers residency; measured C3 +1%, C5 -7%). */
+  int sweep_rhs_pairs;         /* accepted and ignored: the sweeps of complex FP32 factors always take the
+                                  right-hand sides of a wavelength two at a time from the factor entries
+                                  staged in shared memory, each of which is read from memory once. */
   int tensor_offdiag;          /* 1: complex FP32 LU fronts whose update matrices go to the tensor cores
                                   (tensor_form > 0, block-local pivoting) also form L21 = F21 U11^-1 and
                                   U12 = L11^-1 P F12 there, as products with the triangular inverses, and

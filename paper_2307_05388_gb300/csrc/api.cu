@@ -43,20 +43,6 @@ struct LevelList {
   int tqt_off = 0, ntqt = 0;                    // their output tiles
 };
 
-struct TaskList {
-  int off = 0, n = 0;      // int2 (front, first row or column) tasks at d_lists + off
-};
-
-
-// Sweep tasks of one level; index 0 = row tasks (sweeps L, U), 1 = column tasks (U^T, L^T).
-struct SolveList {
-  TaskList tri[2];         // inverse-block products, every front of the level
-  TaskList rect_m[2];      // off-diagonal block split over the m boundary rows/columns
-  TaskList rect_k[2];      // off-diagonal block split over the k pivot rows/columns
-  int kmax = 0;            // shared-memory vector entries the tri launch needs
-  int kbig = 0, mbig = 0;  // largest k and m among fronts with boundary rows
-};
-
 template <typename P>
 cudaError_t dalloc(P** p, size_t bytes) {
   *p = nullptr;
@@ -114,10 +100,20 @@ struct fdfd_ctx {
   unsigned char* d_pivonly = nullptr;   // [full, design][front]: c64 LU panel steps over the pivot block only
   std::vector<unsigned char> h_pivonly;
   std::vector<LevelList> lv_full[3], lv_design[3];   // [0 = c64 LU, 1 = c128 LU, 2 = c64 symmetric form]
-  std::vector<SolveList> lv_solve;
-  // dataflow sweep queues [task type: 0 rows, 1 columns][direction: 0 bottom-up, 1 top-down]
-  struct FlowList { int off = 0, n = 0, uoff = 0, nu = 0, need_all = 0, need_ph1 = 0; } flow[2][2];
-  int flow_vmax = 0;               // shared-memory vector entries of the flow kernel
+  // dataflow sweep queues [0 = c64, 1 = c128][sweep]: units at d_units[] + uoff
+  struct FlowList { size_t uoff = 0; int nu = 0; } flow[2][4];
+  FlowShape flow_shape[2];
+  SweepFront* d_sweepf = nullptr;  // the fronts as the sweeps read them, by level
+  std::vector<SweepFront> h_sweepf;
+  unsigned char* d_meta = nullptr; // index data of the packed fronts
+  std::vector<unsigned char> h_meta;
+  std::vector<size_t> h_moff;      // where record i's index data starts
+  std::vector<int> h_first;        // records of level l: [h_first[l], h_first[l + 1])
+  SweepUnit* d_units[2] = {nullptr, nullptr};
+  std::vector<SweepUnit> h_units[2];
+  int* d_need[2] = {nullptr, nullptr};   // [sweep][all units, phase-1 units][front]
+  std::vector<int> h_need[2];
+  double ent_lower = 0, ent_upper = 0, ent_rect = 0;   // factor entries a sweep reads, per wavelength
   int* d_flow_ctr = nullptr;       // queue head and per-front counters
   int* d_flow_err = nullptr;       // set by a wait that gave up
   // taps of the design-density filter (offsets and weights) for radius tap_radius
@@ -131,7 +127,7 @@ struct fdfd_ctx {
   int ntap = 0;
   double tap_radius = 0;
   int* h_flow_err = nullptr;       // pinned copy
-  int flow_grid[3] = {0, 0, 0};    // persistent CTAs [0 = c64, 1 = c128, 2 = c64 with right-hand sides in pairs]
+  int flow_grid[2] = {0, 0};       // persistent CTAs [0 = c64, 1 = c128]
 
   // coefficients and permittivity
   double2 *d_cxm = nullptr, *d_cxp = nullptr, *d_cym = nullptr, *d_cyp = nullptr;
@@ -148,6 +144,8 @@ struct fdfd_ctx {
   int* d_perm64 = nullptr;
   float2* d_inv32 = nullptr;       // triangular inverses of the pivot blocks
   double2* d_inv64 = nullptr;
+  float2* d_pack32 = nullptr;      // packed off-diagonal blocks of the small fronts
+  double2* d_pack64 = nullptr;
   float* d_growth = nullptr;
   float* d_growth_max = nullptr;
   int* d_swp = nullptr;            // panel row-swap scratch
@@ -256,6 +254,12 @@ struct Prof {
 void free_plan_device(fdfd_ctx* c) {
   free_ptr(c->d_fronts); free_ptr(c->d_children); free_ptr(c->d_idx); free_ptr(c->d_inv);
   free_ptr(c->d_orig_ptr); free_ptr(c->d_orig_col); free_ptr(c->d_orig_code); free_ptr(c->d_lists);
+  free_ptr(c->d_sweepf); free_ptr(c->d_meta);
+  c->d_sweepf = nullptr; c->d_meta = nullptr;
+  for (int i = 0; i < 2; ++i) {
+    free_ptr(c->d_units[i]); free_ptr(c->d_need[i]);
+    c->d_units[i] = nullptr; c->d_need[i] = nullptr;
+  }
   c->d_fronts = nullptr; c->d_children = c->d_idx = c->d_inv = c->d_orig_ptr = c->d_orig_col = nullptr;
   c->d_orig_code = c->d_lists = nullptr;
   free_ptr(c->d_tcf); free_ptr(c->d_tct); free_ptr(c->d_tcws); free_ptr(c->d_tcpart); free_ptr(c->d_pivonly);
@@ -266,8 +270,8 @@ void free_plan_device(fdfd_ctx* c) {
 
 void free_factor(fdfd_ctx* c) {
   free_ptr(c->d_store32); free_ptr(c->d_store64); free_ptr(c->d_perm32); free_ptr(c->d_perm64);
-  free_ptr(c->d_inv32); free_ptr(c->d_inv64);
-  c->d_inv32 = nullptr; c->d_inv64 = nullptr;
+  free_ptr(c->d_inv32); free_ptr(c->d_inv64); free_ptr(c->d_pack32); free_ptr(c->d_pack64);
+  c->d_inv32 = nullptr; c->d_inv64 = nullptr; c->d_pack32 = nullptr; c->d_pack64 = nullptr;
   free_ptr(c->d_growth);
   free_ptr(c->d_swp);
   c->d_swp = nullptr;
@@ -324,6 +328,223 @@ fdfd_status upload(fdfd_ctx* ctx, P** dst, const std::vector<P>& v) {
   if (!v.empty())
     CK(cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(P), cudaMemcpyHostToDevice, ctx->stream));
   return FDFD_OK;
+}
+
+// Sweeps of problems with 320 thousand unknowns or more (over all wavelengths) are bound by
+// throughput: two CTAs per SM, so that more units are in flight.  Smaller ones are bound by the chain
+// of levels: one CTA with buffers twice as large, so that more fronts run whole.  Measured, two CTAs
+// against one, L sweep: 713 x 259 with three wavelengths (554 thousand) 190 against 258 us, 640 x 480
+// with two (614 thousand) 211 against 275 us; 540 x 540 with eight sources (292 thousand, U^T) 605
+// against 523 us, 100 x 100 54 against 43 us; 340 x 340 is a tie (112 and 118 us).
+bool flow_wide(const fdfd_ctx* ctx) { return (long long)ctx->nx * ctx->ny * ctx->n_omega >= 320000; }
+// bytes of one of a CTA's two buffers (with the static arrays the CTAs fill an SM's shared memory)
+constexpr int kFlowSmemWide = 51 * 1024, kFlowSmemNarrow = 104 * 1024;
+constexpr int kFlowCtasNarrow = 1;
+
+long long round16(long long b) { return (b + 15) / 16 * 16; }
+
+// The sweeps' records of the fronts and the packed fronts' index data (sweep.h), in sweep order.
+void build_records(fdfd_ctx* ctx) {
+  const Plan& p = ctx->plan;
+  const size_t nf = p.fronts.size();
+  std::vector<SweepFront>& recs = ctx->h_sweepf;
+  std::vector<unsigned char>& meta = ctx->h_meta;
+  std::vector<size_t>& moff = ctx->h_moff;
+  std::vector<int>& first = ctx->h_first;
+  recs.clear();
+  recs.reserve(nf);
+  moff.assign(nf + 1, 0);
+  first.assign(p.n_levels + 1, 0);
+  size_t bytes = 0;
+  for (const FrontDesc& d : p.fronts)
+    if (d.n <= kPackMaxN) bytes += meta_bytes(d.n);
+  meta.assign(bytes, 0);
+  ctx->ent_lower = ctx->ent_upper = ctx->ent_rect = 0;
+  for (int f : p.sweep_order) {
+    const FrontDesc& d = p.fronts[f];
+    SweepFront r;
+    r.k = d.k; r.m = d.m; r.ld = d.ld; r.ldk = d.ldk;
+    r.st_off = d.st_off; r.iv_off = d.iv_off; r.pk_off = d.pk_off; r.v_off = d.v_off;
+    r.u0 = r.u1 = 0;
+    r.inv0 = r.inv1 = r.dep0 = r.dep1 = -1;
+    if (d.nchild > 0) {
+      const int c = p.children[d.child0];
+      r.dep0 = c; r.inv0 = p.fronts[c].inv_off; r.u0 = p.fronts[c].v_off + p.fronts[c].k;
+    }
+    if (d.nchild > 1) {
+      const int c = p.children[d.child0 + 1];
+      r.dep1 = c; r.inv1 = p.fronts[c].inv_off; r.u1 = p.fronts[c].v_off + p.fronts[c].k;
+    }
+    r.parent = d.parent; r.f = f; r.idx_off = d.idx_off; r.piv_off = d.piv_off;
+    const size_t i = recs.size();
+    recs.push_back(r);
+    first[d.level + 1] = (int)i + 1;
+    moff[i + 1] = moff[i];
+    if (d.n <= kPackMaxN) {
+      unsigned char* o = meta.data() + moff[i];
+      std::memcpy(o, &r, sizeof(r));
+      std::memcpy(o + 96, &p.idx[d.idx_off], sizeof(int) * d.n);
+      unsigned* s = reinterpret_cast<unsigned*>(o + 96 + sizeof(int) * d.n);
+      for (int t = 0; t < d.n; ++t)
+        s[t] = (r.inv0 >= 0 ? (unsigned)p.inv[r.inv0 + t] & 0xffffu : 0xffffu) |
+               (r.inv1 >= 0 ? (unsigned)p.inv[r.inv1 + t] & 0xffffu : 0xffffu) << 16;
+      moff[i + 1] += meta_bytes(d.n);
+    }
+    ctx->ent_lower += 0.5 * d.k * (d.k - 1.0);
+    ctx->ent_upper += 0.5 * d.k * (d.k + 1.0);
+    ctx->ent_rect += (double)d.k * d.m;
+  }
+}
+
+// The sweeps' units for one precision (0 = c64, 1 = c128).  Per level: whole small fronts a warp
+// each; fronts whose factor blocks and vectors fit a buffer, one unit each; the others in units of
+// rows (L, U) or columns (U^T, L^T) whose parts fit.
+void build_units(fdfd_ctx* ctx, int prec) {
+  const Plan& p = ctx->plan;
+  const std::vector<SweepFront>& recs = ctx->h_sweepf;
+  const std::vector<size_t>& moff = ctx->h_moff;
+  const int nf = (int)recs.size(), nl = p.n_levels;
+  int nsm = 1, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    nsm = 1;
+  const int es = prec == 0 ? 8 : 16, nv = prec == 0 ? 2 : 1;   // right-hand sides a unit has vectors for
+  const int packed_n = lu_small_max_n(es), nwarp = kFlowThreads / 32;
+  const bool wide = prec == 0 && flow_wide(ctx);
+  const long long ctas = (long long)nsm * (wide ? kFlowWideCtas : kFlowCtasNarrow);
+  auto packed = [&](int r) { return recs[r].k + recs[r].m <= packed_n; };
+  auto fac_bytes = [&](int r) { return (long long)pack_block(recs[r].m, recs[r].k) * es; };
+  auto vec_bytes = [&](int r) { return round16((long long)(recs[r].m + 2 * recs[r].k) * nv * es); };
+  // every packed front fits whole (the small LU writes no other form)
+  long long need = wide ? kFlowSmemWide : kFlowSmemNarrow;
+  for (int r = 0; r < nf; ++r)
+    if (packed(r)) need = std::max(need, (long long)(moff[r + 1] - moff[r]) + fac_bytes(r) + vec_bytes(r));
+  FlowShape& sh = ctx->flow_shape[prec];
+  sh.wide = wide;
+  sh.buffers = 2 * need <= kFlowMaxSmem ? 2 : 1;
+  sh.smem = (int)need;
+  const long long budget = need;
+  // units of the packed fronts, the same in every sweep: level l has [pfirst[l], pfirst[l + 1])
+  std::vector<SweepUnit> punits;
+  std::vector<int> pfirst(nl + 1, 0), pend(nl, 0);
+  for (int l = 0; l < nl; ++l) {
+    const int r0 = ctx->h_first[l], r1 = ctx->h_first[l + 1];
+    int rp = r0, r64 = r0;                               // the level's packed records [r0, rp), n <= kTrimMaxN [r0, r64)
+    while (rp < r1 && packed(rp)) ++rp;
+    while (r64 < rp && recs[r64].k + recs[r64].m <= kTrimMaxN) ++r64;
+    const bool many = (long long)(rp - r0) * ctx->n_omega > 4 * ctas;
+    const int rs = many ? rp : r64;                      // a warp each [r0, rs), a CTA each [rs, rp)
+    for (int r = r0; r < rp;) {
+      const bool small = r < rs;
+      SweepUnit u;
+      std::memset(&u, 0, sizeof(u));
+      long long fac = 0, vs = 0;
+      int cnt = 0;
+      while (r + cnt < (small ? rs : r + 1) && cnt < (small ? nwarp : 1)) {
+        const long long f2 = fac + fac_bytes(r + cnt), v2 = std::max(vs, vec_bytes(r + cnt));
+        if (cnt && (long long)(moff[r + cnt + 1] - moff[r]) + f2 + (cnt + 1) * v2 > budget) break;
+        u.off[cnt] = (unsigned short)((moff[r + cnt] - moff[r]) / 16);
+        fac = f2;
+        vs = v2;
+        ++cnt;
+      }
+      u.rec = (int)(moff[r] / 16);
+      u.kind = (small ? kUnitSmall : kUnitPacked) | (cnt << 8);
+      u.r0 = (int)(moff[r + cnt] - moff[r]);
+      u.cnt = (int)fac;
+      u.fac = recs[r].pk_off;
+      u.vslice = (int)vs;
+      punits.push_back(u);
+      r += cnt;
+    }
+    pend[l] = rp;
+    pfirst[l + 1] = (int)punits.size();
+  }
+  std::vector<SweepUnit>& units = ctx->h_units[prec];
+  std::vector<int>& need_lists = ctx->h_need[prec];
+  units.clear();
+  need_lists.assign((size_t)8 * nf, 0);                  // per sweep: all units of each front, its phase-1 units
+  for (int sweep = 0; sweep < 4; ++sweep) {
+    const bool up = sweep == 0 || sweep == 2, rows = sweep < 2;
+    auto& fl = ctx->flow[prec][sweep];
+    fl.uoff = units.size();
+    int* all = need_lists.data() + (size_t)(2 * sweep) * nf;
+    int* ph1 = all + nf;
+    for (int r = 0; r < nf; ++r)
+      if (packed(r)) all[recs[r].f] = 1;
+    std::vector<int> fronts, large;
+    for (int li = 0; li < nl; ++li) {
+      const int l = up ? li : nl - 1 - li;
+      fronts.clear();
+      large.clear();
+      long long lines[2] = {0, 0};    // rows or columns of the level's large fronts
+      for (int r = pend[l]; r < ctx->h_first[l + 1]; ++r) {
+        const SweepFront& d = recs[r];
+        const StageGeom g = stage_geom(es, sweep, true, d.k, d.ld, d.ldk, 0, up ? d.m : d.k, 0, up ? d.k : d.m, kFlowThreads);
+        const long long fp = (long long)sizeof(SweepFront) + (long long)d.k * d.ldk * es + stage_bytes(g, es) + vec_bytes(r);
+        if (fp <= budget) {
+          fronts.push_back(r);
+        } else {
+          large.push_back(r);
+          lines[0] += d.k;
+          lines[1] += up ? d.m : d.k;
+        }
+      }
+      auto add = [&](int rec, int kind, int r0, int cnt, int part) {
+        SweepUnit u;
+        std::memset(&u, 0, sizeof(u));
+        u.rec = rec; u.kind = kind; u.r0 = r0; u.cnt = cnt; u.vslice = part;
+        units.push_back(u);
+        all[recs[rec].f]++;
+      };
+      auto put_whole = [&]() {
+        units.insert(units.end(), punits.begin() + pfirst[l], punits.begin() + pfirst[l + 1]);
+        for (int r : fronts) add(r, kUnitFront, 0, 0, 0);
+      };
+      auto put_large = [&](bool rect, bool phase1) {
+        const long long share = lines[rect] * ctx->n_omega / ctas;    // lines per CTA, so that a short level still spreads
+        for (int r : large) {
+          const SweepFront& d = recs[r];
+          if (rect && d.m == 0) continue;
+          const int len = rect && up ? d.m : d.k;          // rows (columns) to cover
+          // up to 64 lines to a unit, and to the level's share of a CTA; the contraction in the fewest
+          // equal parts that fit a buffer
+          for (int s0 = 0, c; s0 < len; s0 += c) {
+            c = rows ? 8 : 16;
+            while (2 * c <= 64 && 2 * c <= share) c *= 2;
+            c = std::min(c, len - s0);
+            const UnitRange ur = unit_range(sweep, rect, d.k, d.m, s0, c);
+            const int total = ur.hi - ur.lo;
+            int part = 8;
+            for (int np = 1; np <= total; ++np) {
+              part = ((total + np - 1) / np + 7) / 8 * 8;
+              const StageGeom g = stage_geom(es, sweep, rect, d.k, d.ld, d.ldk, s0, c, ur.lo,
+                                             std::min(ur.lo + part, ur.hi), kFlowThreads);
+              // (another part's rows may start one entry earlier and their stride be one step longer)
+              if ((long long)sizeof(SweepFront) + round16((long long)(part + 2 + c) * nv * es) +
+                      (long long)g.rows * (g.stride + 2) * es <= budget)
+                break;
+            }
+            add(r, rect ? kUnitRect : kUnitTri, s0, c, part);
+            if (phase1) ph1[d.f]++;
+          }
+        }
+      };
+      if (up) { put_whole(); put_large(false, true); put_large(true, false); }
+      else { put_large(true, true); put_whole(); put_large(false, false); }
+    }
+    fl.nu = (int)(units.size() - fl.uoff);
+  }
+}
+
+template <typename P>
+fdfd_status upload(fdfd_ctx* ctx, P** dst, const std::vector<P>& v);
+
+// The units of one precision, built and uploaded when its factors are first asked for.
+fdfd_status ensure_units(fdfd_ctx* ctx, int prec) {
+  if (ctx->d_units[prec]) return FDFD_OK;
+  build_units(ctx, prec);
+  CKS(upload(ctx, &ctx->d_need[prec], ctx->h_need[prec]));
+  return upload(ctx, &ctx->d_units[prec], ctx->h_units[prec]);
 }
 
 // Uploads the plan and builds the per-level launch lists.  The host vectors
@@ -524,148 +745,11 @@ fdfd_status upload_plan(fdfd_ctx* ctx) {
       }
     }
   }
-  ctx->lv_solve.assign(L, SolveList{});
-  // task lists (front, first row/column): [0] row tasks, [1] column tasks.
-  // A small or medium front is one whole-front task (front | bit 31; y = 0 for
-  // one warp, 1 for one CTA); a large front is split into row or column tasks
-  // in both directions.
-  const int whole_n = flow_whole_max_n();   // fronts swept whole by one warp
-  const int cta_n = flow_cta_max_n();       // ... or by one CTA
-  auto small = [cta_n](const FrontDesc& d) { return d.n <= cta_n; };
-  // Row tasks of a level with many of them take two rows per warp (kSweepTaskTall,
-  // flagged in the task word): fewer, longer tasks with more loads in flight.
-  int sweep_nsm = 0;
-  {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sweep_nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sweep_nsm = 1;
-  }
-  auto tall_level = [&](int l) {
-    long long cnt = 0;
-    for (int f : p.level_fronts[l]) {
-      const FrontDesc& d = p.fronts[f];
-      if (small(d)) continue;
-      cnt += (d.k + 7) / 8 + (d.m + 7) / 8;
-    }
-    return cnt * ctx->n_omega >= 16LL * sweep_nsm;
-  };
-  auto add_tasks = [&](TaskList& tl, int l, bool rect, bool over_m, int step) {
-    if (lists.size() % 2) lists.push_back(0);   // int2 task arrays stay 8-byte aligned
-    tl.off = (int)lists.size();
-    const bool tall = step == sweep_row_block() && tall_level(l);
-    const int st = tall ? 2 * step : step;
-    const unsigned flag = tall ? (unsigned)kSweepTaskTall : 0u;
-    for (int f : p.level_fronts[l]) {
-      const FrontDesc& d = p.fronts[f];
-      if (small(d)) {
-        if (!rect) {
-          lists.push_back((int)(0x80000000u | (unsigned)f));
-          lists.push_back(d.n <= whole_n ? 0 : 1);
-          tl.n++;
-        }
-        continue;
-      }
-      if (rect && d.m == 0) continue;
-      const int len = over_m ? d.m : d.k;
-      for (int s0 = 0; s0 < len; s0 += st) { lists.push_back((int)(flag | (unsigned)f)); lists.push_back(s0); tl.n++; }
-    }
-  };
-  const int steps[2] = {sweep_row_block(), sweep_col_block()};
-  for (int l = 0; l < L; ++l) {
-    SolveList& sl = ctx->lv_solve[l];
-    for (int t = 0; t < 2; ++t) {
-      add_tasks(sl.tri[t], l, false, false, steps[t]);     // inverse blocks (whole small fronts)
-      add_tasks(sl.rect_m[t], l, true, true, steps[t]);    // off-diagonal block, over boundary rows/cols
-      add_tasks(sl.rect_k[t], l, true, false, steps[t]);   // off-diagonal block, over pivot rows/cols
-    }
-    for (int f : p.level_fronts[l]) {
-      const FrontDesc& d = p.fronts[f];
-      sl.kmax = std::max(sl.kmax, small(d) ? d.n + d.k : d.k);   // shared-memory vectors of the tri launch
-      if (!small(d) && d.m > 0) {
-        sl.mbig = std::max(sl.mbig, d.m);
-        sl.kbig = std::max(sl.kbig, d.k);
-      }
-    }
-    ctx->flow_vmax = std::max({ctx->flow_vmax, sl.kmax, sl.kbig, sl.mbig});
-  }
-  // Dataflow queues: the same tasks as the level lists, in dependency order,
-  // off-diagonal tasks tagged with bit 30; per level the whole small fronts
-  // first, in units of up to 8 (one warp each), then the whole medium fronts
-  // (one CTA each), then the large fronts' tasks (one unit each) in phase
-  // order; per-front task counts beside them.
-  const int nf = (int)p.fronts.size();
-  for (int t = 0; t < 2; ++t) {
-    for (int dir = 0; dir < 2; ++dir) {
-      auto& fl = ctx->flow[t][dir];
-      fl = fdfd_ctx::FlowList{};                 // the plan may be uploaded again (plain mode)
-      std::vector<int> all(nf, 0), ph1(nf, 0);
-      std::vector<int> tasks, units;
-      auto put_unit = [&](int first, int y) { units.push_back(first); units.push_back(y); };
-      auto put_whole = [&](const SolveList& sl) {
-        int first = -1, cnt = 0;
-        for (int i = 0; i < sl.tri[t].n; ++i) {
-          const int code = lists[sl.tri[t].off + 2 * i];
-          if (code >= 0 || lists[sl.tri[t].off + 2 * i + 1] != 0) continue;   // not a small front
-          const int f = code & kSweepFrontMask;
-          if (cnt == 0) first = (int)tasks.size() / 2;
-          tasks.push_back(code); tasks.push_back(0);
-          all[f]++;
-          if (++cnt == 8) { put_unit(first, (int)(0x80000000u | 8u)); cnt = 0; }
-        }
-        if (cnt) put_unit(first, (int)(0x80000000u | (unsigned)cnt));
-        for (int i = 0; i < sl.tri[t].n; ++i) {               // whole medium fronts, one unit each
-          const int code = lists[sl.tri[t].off + 2 * i];
-          if (code >= 0 || lists[sl.tri[t].off + 2 * i + 1] != 1) continue;
-          put_unit((int)tasks.size() / 2, 1);
-          tasks.push_back(code); tasks.push_back(1);
-          all[code & kSweepFrontMask]++;
-        }
-      };
-      auto put_tri = [&](const SolveList& sl) {
-        for (int i = 0; i < sl.tri[t].n; ++i) {
-          const int code = lists[sl.tri[t].off + 2 * i], s0 = lists[sl.tri[t].off + 2 * i + 1];
-          if (code < 0) continue;                            // whole small front
-          put_unit((int)tasks.size() / 2, 1);
-          tasks.push_back(code); tasks.push_back(s0);
-          all[code & kSweepFrontMask]++;
-          if (dir == 0) ph1[code & kSweepFrontMask]++;
-        }
-      };
-      auto put_rect = [&](const TaskList& tl) {
-        for (int i = 0; i < tl.n; ++i) {
-          const int code = lists[tl.off + 2 * i], s0 = lists[tl.off + 2 * i + 1];
-          const int f = code & kSweepFrontMask;
-          put_unit((int)tasks.size() / 2, 1);
-          tasks.push_back((int)(0x40000000u | (unsigned)code)); tasks.push_back(s0);
-          all[f]++;
-          if (dir == 1) ph1[f]++;
-        }
-      };
-      if (dir == 0) {
-        for (int l = 0; l < L; ++l) {
-          put_whole(ctx->lv_solve[l]); put_tri(ctx->lv_solve[l]); put_rect(ctx->lv_solve[l].rect_m[t]);
-        }
-      } else {
-        for (int l = L - 1; l >= 0; --l) {
-          put_rect(ctx->lv_solve[l].rect_k[t]); put_whole(ctx->lv_solve[l]); put_tri(ctx->lv_solve[l]);
-        }
-      }
-      if (lists.size() % 2) lists.push_back(0);
-      fl.off = (int)lists.size();
-      fl.n = (int)tasks.size() / 2;
-      lists.insert(lists.end(), tasks.begin(), tasks.end());
-      fl.uoff = (int)lists.size();
-      fl.nu = (int)units.size() / 2;
-      lists.insert(lists.end(), units.begin(), units.end());
-      fl.need_all = (int)lists.size();
-      lists.insert(lists.end(), all.begin(), all.end());
-      fl.need_ph1 = (int)lists.size();
-      lists.insert(lists.end(), ph1.begin(), ph1.end());
-    }
-  }
+  build_records(ctx);
   ctx->h_lists.swap(lists);
   CKS(upload(ctx, &ctx->d_lists, ctx->h_lists));
+  CKS(upload(ctx, &ctx->d_sweepf, ctx->h_sweepf));
+  CKS(upload(ctx, &ctx->d_meta, ctx->h_meta));
   ctx->h_tcf.swap(tcf);
   ctx->h_tct.swap(tct);
   if (!ctx->h_tcf.empty()) {
@@ -740,6 +824,7 @@ DevCoef dev_coef(const fdfd_ctx* c) {
 
 fdfd_status ensure_store(fdfd_ctx* ctx, int prec) {
   const Plan& p = ctx->plan;
+  CKS(ensure_units(ctx, prec));
   const size_t nfr = p.fronts.size();
   if (!ctx->d_growth) CK(dalloc(&ctx->d_growth, sizeof(float) * nfr * ctx->n_omega));
   if (!ctx->d_swp)
@@ -751,11 +836,13 @@ fdfd_status ensure_store(fdfd_ctx* ctx, int prec) {
     CK(dalloc(&ctx->d_store32, sizeof(float2) * (size_t)p.store_total * ctx->n_omega));
     CK(dalloc(&ctx->d_perm32, sizeof(int) * (size_t)std::max(1, p.perm_total) * ctx->n_omega));
     CK(dalloc(&ctx->d_inv32, sizeof(float2) * (size_t)p.inv_total * ctx->n_omega));
+    CK(dalloc(&ctx->d_pack32, sizeof(float2) * (size_t)std::max<long long>(2, 2 * p.pack_total) * ctx->n_omega));
   }
   if (prec == 1 && !ctx->d_store64) {
     CK(dalloc(&ctx->d_store64, sizeof(double2) * (size_t)p.store_total * ctx->n_omega));
     CK(dalloc(&ctx->d_perm64, sizeof(int) * (size_t)std::max(1, p.perm_total) * ctx->n_omega));
     CK(dalloc(&ctx->d_inv64, sizeof(double2) * (size_t)p.inv_total * ctx->n_omega));
+    CK(dalloc(&ctx->d_pack64, sizeof(double2) * (size_t)std::max<long long>(2, 2 * p.pack_total) * ctx->n_omega));
   }
   return FDFD_OK;
 }
@@ -783,6 +870,8 @@ fdfd_status factor_levels(fdfd_ctx* ctx, bool design_only, int w0 = 0, int nw = 
   fa.swp_stride = std::max(1, ctx->max_nlarge);
   fa.istore = prec == 0 ? (void*)ctx->d_inv32 : (void*)ctx->d_inv64;
   fa.istore_stride = p.inv_total;
+  fa.pack = prec == 0 ? (void*)ctx->d_pack32 : (void*)ctx->d_pack64;
+  fa.pack_stride = 2 * p.pack_total;
   fa.sym = sym ? 1 : 0;
   const int form = sym ? 2 : prec;
   // complex64 LU with block-local pivoting: the fronts whose update matrices go to the
@@ -1020,22 +1109,12 @@ fdfd_status factor_levels(fdfd_ctx* ctx, bool design_only, int w0 = 0, int nw = 
   return FDFD_OK;
 }
 
-// Sweeps of problems with at least 2^20 unknowns over all wavelengths run the
-// flow-kernel variant with six resident CTAs per SM (more loads in flight);
-// smaller ones keep four, with more registers per thread for their
-// latency-bound tasks.
-bool flow_wide(const fdfd_ctx* ctx) { return (long long)ctx->nx * ctx->ny * ctx->n_omega >= (1LL << 20); }
-
 fdfd_status ensure_ws(fdfd_ctx* ctx, int nrhs) {
   if (ctx->ws_nrhs >= nrhs) return FDFD_OK;
   free_ws(ctx);
   const size_t S = (size_t)ctx->n_omega * nrhs;
   CK(dalloc(&ctx->d_vb, sizeof(double2) * S * (size_t)ctx->plan.vec_total));
   CK(dalloc(&ctx->d_flow_ctr, sizeof(int) * (1 + 2 * (size_t)ctx->n_omega * ctx->plan.fronts.size())));
-  int nsm = 0;
-  CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-  for (int v = 0; v < 3; ++v)
-    ctx->flow_grid[v] = nsm * flow_blocks_per_sm(v == 1 ? 16 : 8, std::max(1, ctx->flow_vmax), flow_wide(ctx), v == 2);
   ctx->ws_nrhs = nrhs;
   return FDFD_OK;
 }
@@ -1053,6 +1132,8 @@ SolveLaunch solve_launch(const fdfd_ctx* ctx, void* vb, int nrhs, int w0, int nw
   sa.perm_stride = std::max(1, p.perm_total);
   sa.istore = prec == 0 ? (const void*)ctx->d_inv32 : (const void*)ctx->d_inv64;
   sa.istore_stride = p.inv_total;
+  sa.pack = prec == 0 ? (const void*)ctx->d_pack32 : (const void*)ctx->d_pack64;
+  sa.pack_stride = 2 * p.pack_total;
   sa.vb = vb;
   sa.vec_stride = p.vec_total;
   sa.n_omega = nw < 0 ? ctx->n_omega : nw;
@@ -1070,11 +1151,10 @@ SolveLaunch solve_launch(const fdfd_ctx* ctx, void* vb, int nrhs, int w0, int nw
 
 // Persistent CTAs of the dataflow sweep for precision prec (host queries only).
 int flow_grid(fdfd_ctx* ctx, int prec) {
-  if (ctx->flow_grid[prec] > 0) return ctx->flow_grid[prec];   // prec 2: the paired-RHS variant of c64
+  if (ctx->flow_grid[prec] > 0) return ctx->flow_grid[prec];
   int nsm = 0;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || nsm <= 0) nsm = 1;
-  ctx->flow_grid[prec] = nsm * flow_blocks_per_sm(prec == 1 ? 16 : 8, std::max(1, ctx->flow_vmax), flow_wide(ctx),
-                                                  prec == 2);
+  ctx->flow_grid[prec] = nsm * flow_blocks_per_sm(prec == 1 ? 16 : 8, ctx->flow_shape[prec]);
   return ctx->flow_grid[prec];
 }
 
@@ -1090,81 +1170,40 @@ fdfd_status sweep_pair(fdfd_ctx* ctx, const SolveLaunch& sa, int transpose, cons
   // gathered, A^T x = b with D x written), 1 / d taken between them
   const bool sym = sa.sym_mid != 0;
   const int fwd = sym ? 0 : (transpose ? 2 : 0), bwd = sym ? 3 : (transpose ? 3 : 1);
-  const double es = sizeof(T), nsys = (double)sa.n_omega * sa.nr;
-  int tt = transpose ? 1 : 0;                             // row tasks (L, U) or column tasks (U^T, L^T)
-  int step = tt ? sweep_col_block() : sweep_row_block();
-  // algorithmic work: every entry of the swept triangle (and of the off-diagonal
-  // block) read once per right-hand side, 8 flops per entry, plus the vectors
-  auto tri_work = [&](const TaskList& tl, bool lower, double* fl, double* by) {
-    *fl = *by = 0;
-    if (!ctx->prof_on) return;
-    for (int t = 0; t < tl.n; ++t) {
-      const int e = ctx->h_lists[tl.off + 2 * t];
-      const FrontDesc& d = p.fronts[e & kSweepFrontMask];
-      const bool whole = e < 0;
-      const int b0 = whole ? 0 : ctx->h_lists[tl.off + 2 * t + 1];
-      const int rows = (e & kSweepTaskTall) ? 2 * step : step;
-      const int b1 = whole ? d.k : std::min(d.k, b0 + rows);
-      double ent = 0;   // entries of this task's rows (or columns) inside the triangle
-      for (int r = b0; r < b1; ++r) ent += lower ? r : (d.k - r);
-      if (whole) ent += (double)d.k * d.m;   // whole-front tasks also do the off-diagonal block
-      *fl += 8.0 * ent * nsys;
-      *by += es * (ent + (b1 - b0)) * nsys;
-    }
-  };
-  auto rect_work = [&](const TaskList& tl, bool over_m, double* fl, double* by) {
-    *fl = *by = 0;
-    if (!ctx->prof_on) return;
-    for (int t = 0; t < tl.n; ++t) {
-      const int e = ctx->h_lists[tl.off + 2 * t];
-      const FrontDesc& d = p.fronts[e & kSweepFrontMask];
-      const int s0 = ctx->h_lists[tl.off + 2 * t + 1];
-      const double rows = std::min((e & kSweepTaskTall) ? 2 * step : step, (over_m ? d.m : d.k) - s0);
-      const double other = over_m ? d.k : d.m;
-      *fl += 8.0 * rows * other * nsys;
-      *by += es * rows * (other + 1) * nsys;
-    }
-  };
-  const int* dl = ctx->d_lists;
+  const double es = sizeof(T);
   const size_t ctr_bytes = sizeof(int) * (1 + 2 * (size_t)sa.n_omega * p.fronts.size());
-  // complex64 factors with an even number of right-hand sides per wavelength: the paired variant
-  const bool pairs = prec == 0 && ctx->opt.sweep_rhs_pairs && sa.nr >= 2 && sa.nr % 2 == 0;
-  const int grid_max = flow_grid(ctx, pairs ? 2 : prec);
-  for (int dir = 0; dir < 2; ++dir) {
+  const int grid_max = flow_grid(ctx, prec);
+  for (int step = 0, groups = (sa.nr + kFlowMaxRhs - 1) / kFlowMaxRhs; step < 2 * groups; ++step) {
+    const int dir = step / groups, rg = step % groups * kFlowMaxRhs;   // up to kFlowMaxRhs right-hand sides at a time
     SolveLaunch sd = sa;
+    sd.r0 = sa.r0 + rg;
+    sd.nr = std::min(kFlowMaxRhs, sa.nr - rg);
+    const double nsys = (double)sd.n_omega * sd.nr;
     if (sym) {
-      tt = dir;                                            // L: row tasks; L^T: column tasks
-      step = tt ? sweep_col_block() : sweep_row_block();
       sd.sym_in = (dir == 0 && !transpose) ? 1 : 0;
       sd.sym_out = (dir == 1 && transpose) ? 1 : 0;
       sd.sym_mid = dir == 1 ? 1 : 0;
     }
-    const auto& fq = ctx->flow[tt][dir];
-    double fl = 0, by = 0;
-    for (int l = 0; l < p.n_levels; ++l) {
-      const SolveList& sl = ctx->lv_solve[l];
-      double f1, b1;
-      tri_work(sl.tri[tt], sym ? true : (dir == 0 ? !transpose : transpose), &f1, &b1);
-      fl += f1; by += b1;
-      rect_work(dir == 0 ? sl.rect_m[tt] : sl.rect_k[tt], dir == 0, &f1, &b1);
-      fl += f1; by += b1;
-    }
+    const int sweep = dir == 0 ? fwd : bwd;
+    const auto& fq = ctx->flow[prec][sweep];
+    // algorithmic work: every entry of the swept triangle and of the off-diagonal block once per
+    // right-hand side, 8 flops per entry, plus the vectors
+    const double ent = (sweep == 0 || sweep == 3 ? ctx->ent_lower : ctx->ent_upper) + ctx->ent_rect;
     CK(cudaMemsetAsync(ctr, 0, ctr_bytes, s));
     FlowQueue q;
-    q.tasks = reinterpret_cast<const int2*>(dl + fq.off);
-    q.units = reinterpret_cast<const int2*>(dl + fq.uoff);
+    q.fronts = ctx->d_sweepf;
+    q.meta = ctx->d_meta;
+    q.units = ctx->d_units[prec] + fq.uoff;
     q.nunits = fq.nu;
     q.ctr = ctr;
-    q.need_all = dl + fq.need_all;
-    q.need_ph1 = dl + fq.need_ph1;
+    q.need_all = ctx->d_need[prec] + (size_t)(2 * sweep) * p.fronts.size();
+    q.need_ph1 = q.need_all + p.fronts.size();
     q.err = ctx->d_flow_err;
     q.n_fronts = (int)p.fronts.size();
-    const int grid = std::max(1, std::min(grid_max, fq.nu * sa.n_omega));
-    const int kind = sym ? (dir == 0 ? PK_SWEEP_L : PK_SWEEP_LT)
-                         : (dir == 0 ? (transpose ? PK_SWEEP_UT : PK_SWEEP_L) : (transpose ? PK_SWEEP_LT : PK_SWEEP_U));
-    Prof pr(ctx, kind, fl, by);
-    launch_sweep_flow<T>(sd, dir == 0 ? fwd : bwd, q, std::max(1, ctx->flow_vmax), grid, in, out, s, flow_wide(ctx),
-                         pairs);
+    const int grid = (int)std::max<long long>(1, std::min<long long>(grid_max, (long long)fq.nu * sa.n_omega));
+    static const int kinds[4] = {PK_SWEEP_L, PK_SWEEP_U, PK_SWEEP_UT, PK_SWEEP_LT};
+    Prof pr(ctx, kinds[sweep], 8.0 * ent * nsys, es * (ent + (double)p.vec_total) * nsys);
+    launch_sweep_flow<T>(sd, sweep, q, ctx->flow_shape[prec], grid, in, out, s);
   }
   CK(cudaGetLastError());
   return FDFD_OK;
@@ -1477,6 +1516,9 @@ fdfd_status settle_growth(fdfd_ctx* ctx, bool* fell_back = nullptr, bool* repivo
   if (fell_back) *fell_back = true;
   return refactor_f64(ctx);
 }
+
+// row stride of a front as the introspection calls show it
+int front_ld(const FrontDesc& d) { return (d.n + 3) / 4 * 4; }
 
 fdfd_status solve_direct(fdfd_ctx* ctx, const double* b_dev, double* x_dev, int nrhs, int transpose,
                          bool* handled);
@@ -1930,7 +1972,7 @@ fdfd_status fdfd_plan_sizes(fdfd_ctx* ctx, int* n_host, int* ld_host, int* ldk_h
   const Plan& p = ctx->plan;
   for (size_t f = 0; f < p.fronts.size(); ++f) {
     if (n_host) n_host[f] = p.fronts[f].n;
-    if (ld_host) ld_host[f] = p.fronts[f].ld;
+    if (ld_host) ld_host[f] = front_ld(p.fronts[f]);
     if (ldk_host) ldk_host[f] = p.fronts[f].ldk;
   }
   return FDFD_OK;
@@ -1963,12 +2005,56 @@ fdfd_status fdfd_front_copy(fdfd_ctx* ctx, int w, int f, void* front_host, void*
   const char* st = f64 ? reinterpret_cast<const char*>(ctx->d_store64) : reinterpret_cast<const char*>(ctx->d_store32);
   const char* iv = f64 ? reinterpret_cast<const char*>(ctx->d_inv64) : reinterpret_cast<const char*>(ctx->d_inv32);
   CK(cudaStreamSynchronize(ctx->stream));
-  if (front_host)
-    CK(cudaMemcpy(front_host, st + es * ((size_t)w * ctx->plan.store_total + d.st_off), es * (size_t)d.n * d.ld,
-                  cudaMemcpyDeviceToHost));
-  if (inv_host)
-    CK(cudaMemcpy(inv_host, iv + es * ((size_t)w * ctx->plan.inv_total + d.iv_off), es * (size_t)d.k * d.ldk,
-                  cudaMemcpyDeviceToHost));
+  // small fronts: the inverse block, L21 and U12 come from the packed store
+  const bool packed = d.n <= lu_small_max_n((int)es);
+  std::vector<char> pkl, pku;
+  if (packed) {
+    const char* pk = f64 ? reinterpret_cast<const char*>(ctx->d_pack64) : reinterpret_cast<const char*>(ctx->d_pack32);
+    const size_t blk = es * (size_t)pack_block(d.m, d.k), at = 2 * (size_t)w * ctx->plan.pack_total + d.pk_off;
+    pkl.resize(blk);
+    pku.resize(blk);
+    CK(cudaMemcpy(pkl.data(), pk + es * at, blk, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(pku.data(), pk + es * (at + ctx->plan.pack_total), blk, cudaMemcpyDeviceToHost));
+  }
+  if (front_host) {
+    const size_t ld = (size_t)front_ld(d);
+    const size_t wst = (size_t)w * ctx->plan.store_total;
+    char* out = reinterpret_cast<char*>(front_host);
+    if (d.n > kTrimMaxN) {
+      CK(cudaMemcpy(out, st + es * (wst + d.st_off), es * (size_t)d.n * ld, cudaMemcpyDeviceToHost));
+    } else {
+      std::memset(out, 0, es * (size_t)d.n * ld);
+      if (d.m > 0)
+        CK(cudaMemcpy2D(out + es * ((size_t)d.k * ld + d.k), es * ld,
+                        st + es * (size_t)((long long)wst + d.st_off + (long long)d.k * d.ld + d.k), es * d.ld,
+                        es * d.m, d.m, cudaMemcpyDeviceToHost));
+    }
+    if (packed)
+      for (size_t t = 0; t < (size_t)d.m; ++t)
+        for (size_t c = 0; c < (size_t)d.k; ++c) {
+          const size_t e = pack_rect(d.k) + t * pack_stride(d.k) + c;
+          std::memcpy(out + es * ((d.k + t) * ld + c), pkl.data() + es * e, es);
+          std::memcpy(out + es * (c * ld + d.k + t), pku.data() + es * e, es);
+        }
+  }
+  if (inv_host) {
+    char* out = reinterpret_cast<char*>(inv_host);
+    if (!packed) {
+      CK(cudaMemcpy(out, iv + es * ((size_t)w * ctx->plan.inv_total + d.iv_off), es * (size_t)d.k * d.ldk,
+                    cudaMemcpyDeviceToHost));
+    } else {
+      // 1 / d of the symmetric form is on the L side's diagonal, U11^-1 on the U side
+      const bool sym = !f64 && ctx->sym32;
+      std::memset(out, 0, es * (size_t)d.k * d.ldk);
+      for (int t = 0; t < d.k; ++t)
+        for (int i = 0; i + t < d.k; ++i) {
+          const size_t e = (size_t)pack_diag(t, d.k) + i;
+          if (t > 0) std::memcpy(out + es * ((size_t)(i + t) * d.ldk + i), pkl.data() + es * e, es);
+          if (!sym) std::memcpy(out + es * ((size_t)i * d.ldk + i + t), pku.data() + es * e, es);
+          else if (t == 0) std::memcpy(out + es * ((size_t)i * d.ldk + i), pkl.data() + es * e, es);
+        }
+    }
+  }
   return FDFD_OK;
 }
 

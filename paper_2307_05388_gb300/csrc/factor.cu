@@ -176,7 +176,7 @@ __device__ __forceinline__ void warp_argmax(R& v, int& i) {
 // L11\U11 and U12, rows >= k are L21 and the update matrix S in place.
 //
 // Then the triangular inverses, one warp per row, lanes over the columns,
-// from the factors in shared memory into the inverse store:
+// from the factors in shared memory into the packed store (plan.h):
 //   row i of L11^-1: X[i][i] = 1, X[i][l] = -sum_{l < m <= i} X[i][m] L[m][l], m descending;
 //   row i of U11^-1: X[i][c] = (delta_ic - sum_{i <= l < c} X[i][l] U[l][c]) / U[c][c], l ascending.
 // ---------------------------------------------------------------------------
@@ -261,6 +261,18 @@ __device__ __forceinline__ void small_post_column(const T (&x)[RI][RJ], unsigned
   }
   best = __reduce_max_sync(0xffffffffu, best);
   if (lane == 0) *key = best;
+}
+
+// The m rows of a packed block (plan.h): entry (t, c) at t * (k | 1) + c, t < m, c < k (the odd
+// stride's spare column is zero).  Rows of up to 16 entries are written two or four at a time, so
+// that a warp's stores stay full.
+template <typename T, int NWARP, typename Val>
+__device__ __forceinline__ void write_pack_rows(T* __restrict__ B, int m, int k, int warp, int lane, Val val) {
+  const int ks = k | 1;
+  const int lw = ks <= 8 ? 3 : ks <= 16 ? 4 : 5;          // lanes per row: 2^lw
+  const int rpw = 32 >> lw, sub = lane >> lw, c0 = lane & ((1 << lw) - 1);
+  for (int t = warp * rpw + sub; t < m; t += NWARP * rpw)
+    for (int c = c0; c < ks; c += 1 << lw) B[t * ks + c] = c < k ? val(t, c) : czero<T>();
 }
 
 template <typename T, int NWARP, int RI, int RJ, int MINB>
@@ -404,7 +416,8 @@ lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
   __syncthreads();
   // triangular inverses, rows i = warp, warp + NWARP, ...; lane holds columns lane + 32 q (KS slots: k <= 32 KS)
   constexpr int KS = (NMAX + 31) / 32;
-  T* Xg = reinterpret_cast<T*>(a.istore) + (size_t)w * a.istore_stride + d.iv_off;
+  T* Lb = reinterpret_cast<T*>(a.pack) + (size_t)w * a.pack_stride + d.pk_off;   // the front's packed blocks
+  T* Ub = Lb + a.pack_stride / 2;
   const T one = cmk(R(1), R(0));
   T dinv[KS];
 #pragma unroll
@@ -429,7 +442,7 @@ lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
 #pragma unroll
     for (int q = 0; q < KS; ++q) {
       const int l = lane + 32 * q;
-      if (l < i) Xg[(size_t)i * d.ldk + l] = acc[q];
+      if (l < i) Lb[pack_diag(i - l, k) + l] = acc[q];
     }
     // row i of U11^-1, columns c >= i
 #pragma unroll
@@ -447,16 +460,19 @@ lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
 #pragma unroll
     for (int q = 0; q < KS; ++q) {
       const int c = lane + 32 * q;
-      if (c >= i && c < k) Xg[(size_t)i * d.ldk + c] = cmul(acc[q], dinv[q]);
+      if (c >= i && c < k) Ub[pack_diag(c - i, k) + i] = cmul(acc[q], dinv[q]);
     }
   }
-  // the front but its pivot block (U12 in pivot order, L21, S), the permutation, the growth
-  for (int r = warp; r < n; r += NWARP) {
-    const T* Sr = S + (r < k ? s_pm[r] : r) * ls;
+  // the update matrix, the packed off-diagonal blocks, the permutation, the growth
+  for (int r = k + warp; r < n; r += NWARP) {
+    const T* Sr = S + r * ls;
     T* Fr = F + (size_t)r * d.ld;
-    for (int c = (r < k ? k : 0) + lane; c < n; c += 32) Fr[c] = Sr[c];
+    for (int c = k + lane; c < n; c += 32) Fr[c] = Sr[c];
   }
-  int* P = a.perm + (size_t)w * a.perm_stride + d.piv_off;
+  write_pack_rows<T, NWARP>(Lb + pack_rect(k), n - k, k, warp, lane, [&](int t, int c) { return S[(k + t) * ls + c]; });
+  write_pack_rows<T, NWARP>(Ub + pack_rect(k), n - k, k, warp, lane,
+                            [&](int t, int c) { return S[s_pm[c] * ls + k + t]; });
+  int* P = reinterpret_cast<int*>(Lb + pack_perm(n - k, k));
   for (int i = tid; i < k; i += THREADS) P[i] = s_pm[i];
   for (int o = 16; o > 0; o >>= 1) gmax = nanmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
   if (lane == 0) s_red[warp] = gmax;
@@ -495,10 +511,10 @@ template <typename T> struct SmallCfg<T, 96> {
 // complex symmetric (discrete reciprocity), so in the plan's elimination order
 // every front of M factors as F = L diag(d) L^T with no pivoting: L11 unit
 // lower, L21 = F21 L11^-T diag(d)^-1, update matrix S = F22 - L21 diag(d) L21^T.
-// Only lower triangles are formed, updated and stored: the fronts hold L21 and
-// the lower triangle of S (which the parent reads symmetrically), the inverse
-// store holds L11^-1 strictly below the diagonal and 1 / d on it, and the
-// permutation is the identity.  A solve of A x = b is then
+// Only lower triangles are formed, updated and stored: the fronts hold L21 (small
+// ones: the packed store) and the lower triangle of S (which the parent reads
+// symmetrically), the inverse store holds L11^-1 strictly below the diagonal and
+// 1 / d on it, and the permutation is the identity.  A solve of A x = b is then
 //     x = L^-T diag(d)^-1 L^-1 D b   (transpose: A^T x = b gives x = D L^-T diag(d)^-1 L^-1 b),
 // the L and L^T sweeps of the LU path with D and 1 / d applied in between.
 // Small fronts: one CTA per front in shared memory, as lu_small_kernel.  Per
@@ -589,8 +605,8 @@ ldl_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
       gmax = nanmax(gmax, cabs2(l));
     }
   __syncthreads();
-  // L11^-1 rows (as in lu_small_kernel) and 1 / d on the diagonal of the inverse store
-  T* Xg = reinterpret_cast<T*>(a.istore) + (size_t)w * a.istore_stride + d.iv_off;
+  // L11^-1 rows (as in lu_small_kernel) and 1 / d on the diagonal, packed
+  T* Lb = reinterpret_cast<T*>(a.pack) + (size_t)w * a.pack_stride + d.pk_off;
   const T one = cmk(R(1), R(0));
   for (int i = warp; i < k; i += NW) {
     T acc[kSmallSlots];
@@ -607,16 +623,15 @@ ldl_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
 #pragma unroll
     for (int q = 0; q < kSmallSlots; ++q) {
       const int l = lane + 32 * q;
-      if (l < i) Xg[(size_t)i * d.ldk + l] = acc[q];
+      if (l < i) Lb[pack_diag(i - l, k) + l] = acc[q];
     }
-    if (lane == 0) Xg[(size_t)i * d.ldk + i] = crcp(S[i * n + i]);
+    if (lane == 0) Lb[i] = crcp(S[i * n + i]);
   }
-  // rows below the pivots: L21 and the lower triangle of S
-  for (int e = tid; e < (n - k) * n; e += THREADS) {
-    const int r = k + e / n, c = e - (r - k) * n;
-    if (c <= r) F[(size_t)r * d.ld + c] = S[r * n + c];
-  }
-  int* P = a.perm + (size_t)w * a.perm_stride + d.piv_off;
+  // the lower triangle of the update matrix and the packed L21
+  for (int r = k + warp; r < n; r += NW)
+    for (int c = k + lane; c <= r; c += 32) F[(size_t)r * d.ld + c] = S[r * n + c];
+  write_pack_rows<T, NW>(Lb + pack_rect(k), n - k, k, warp, lane, [&](int t, int c) { return S[(k + t) * n + c]; });
+  int* P = reinterpret_cast<int*>(Lb + pack_perm(n - k, k));
   for (int i = tid; i < k; i += THREADS) P[i] = i;
   for (int o = 16; o > 0; o >>= 1) gmax = nanmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
   if (lane == 0) s_red[warp] = gmax;

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "sweep.h"
 
 namespace fdfd {
 
@@ -30,6 +31,8 @@ struct FactorLaunch {
   int swp_stride;          // >= number of fronts in one large-front list
   void* istore;            // triangular inverses (same type as store), [n_omega][istore_stride]
   long long istore_stride;
+  void* pack;              // packed blocks of the small fronts (same type, plan.h), [n_omega][pack_stride]: L half, U half
+  long long pack_stride;
   void* dblk;              // a panel step's diagonal-block factors, [n_omega launched][swp_stride][kDiagBlkElems]
   int sym;                 // 1: symmetric form, M = D A = L diag(d) L^T without pivoting (see factor.cu)
   const unsigned char* pivonly = nullptr;   // per front, or null: 1 = the panel steps factor the k x k pivot block
@@ -132,11 +135,6 @@ cudaError_t factor_init_attributes();   // once per device, before the first fac
 int lu_panel_width(int elem_bytes);
 
 // ---- solve.cu: level-scheduled triangular sweeps ---------------------------
-// sweep task words: front index in the low 29 bits; bit 29 = a row task of
-// 2 x sweep_row_block() rows (two per warp); bit 30 = off-diagonal block; bit 31
-// = a whole small or medium front
-constexpr int kSweepFrontMask = 0x1fffffff;
-constexpr int kSweepTaskTall = 0x20000000;
 struct SolveLaunch {
   DevPlan P;
   const void* store;       // factor storage (T), [n_omega][store_stride]
@@ -145,6 +143,8 @@ struct SolveLaunch {
   int perm_stride;
   const void* istore;      // triangular inverses (T), [n_omega][istore_stride]
   long long istore_stride;
+  const void* pack;        // packed blocks of the small fronts (T, plan.h), [n_omega][pack_stride]: L half, U half
+  long long pack_stride;
   void* vb;                // front vectors (T), [n_sys][vec_stride]
   long long vec_stride;
   int n_omega, nrhs;       // wavelengths launched [w0, w0 + n_omega); nrhs = layout stride
@@ -161,40 +161,38 @@ struct SolveLaunch {
 // back from the output, so they divide D out again.
 // sweep: 0 = L (forward, non-transposed), 1 = U (backward, non-transposed),
 //        2 = U^T (forward of the transpose solve), 3 = L^T (backward of the transpose solve).
-// Large fronts are cut into row tasks of sweep_row_block() rows (sweeps 0, 1)
-// or column tasks of sweep_col_block() columns (sweeps 2, 3).
-int sweep_row_block();
-int sweep_col_block();
 
-// One direction of a sweep pair as a single persistent launch (dataflow over
-// the elimination tree).  tasks: the direction's inverse-block, off-diagonal
-// and whole-front tasks in dependency order (per level: whole small fronts,
-// whole medium fronts, then the large fronts' phase-1 and phase-2 tasks),
-// x = front | 1<<31 (whole front: y = 0 for one warp, y = 1 for one CTA) |
-// 1<<30 (off-diagonal task), y = first row / column.
+// One direction of a sweep pair as a single persistent launch (dataflow over the elimination
+// tree): the sweep's units (sweep.h) in dependency order, per level whole small fronts, whole
+// medium fronts, then the large fronts' phase-1 and phase-2 units; each runs for every launched
+// wavelength.
 struct FlowQueue {
-  const int2* tasks;
-  const int2* units;       // what one CTA takes at a time: (first task, 1) for a large-front task or a
-                           // whole medium front, or
-                           // (first task, 0x80000000 | count) for up to 8 whole small fronts of one level
-  int nunits;              // units; each runs for every launched wavelength
+  const SweepFront* fronts;   // every front, in sweep order
+  const unsigned char* meta;  // index data of the packed fronts, in sweep order
+  const SweepUnit* units;
+  int nunits;
   int* ctr;                // [1 + 2 * n_omega * n_fronts] ints, zero before the launch
-  const int* need_all;     // [n_fronts] tasks of each front in this queue
-  const int* need_ph1;     // [n_fronts] its phase-1 tasks (inverse-block bottom-up, off-diagonal top-down)
+  const int* need_all;     // [n_fronts] units of each front in this queue
+  const int* need_ph1;     // [n_fronts] its phase-1 units (inverse-block bottom-up, off-diagonal top-down)
   int* err;                // set to 1 by a wait that gives up (never cleared by the kernel)
   int n_fronts;
 };
+// A sweep CTA (kFlowThreads working threads): two buffers (one where two do not fit) of `smem` bytes, to which
+// the units are cut with the vectors of two right-hand sides (complex64).
+struct FlowShape {
+  int smem = 0;
+  int buffers = 2;
+  bool wide = false;
+};
+constexpr int kFlowMaxSmem = 208 * 1024;
+constexpr int kFlowMaxRhs = 8;        // right-hand sides of one launch (more: several launches)
+constexpr int kFlowThreads = 256;
+constexpr int kFlowWideCtas = 2;      // per SM
 // in: right-hand sides, out: solutions, both complex128 [systems][n] whatever the
 // factor precision T (converted where the sweeps gather them and store them).
-// wide: the variant that keeps six CTAs resident per SM (large problems) instead of four
-// pairs: allow the paired-RHS variant (complex64 factors, even count per wavelength)
-template <typename T> void launch_sweep_flow(const SolveLaunch& a, int sweep, const FlowQueue& q, int vmax,
-                                             int grid, const void* in, void* out, cudaStream_t s, bool wide,
-                                             bool pairs);
-// pair: the variant that takes right-hand sides in pairs (complex64 factors, even count per wavelength)
-int flow_blocks_per_sm(int elem_bytes, int vmax, bool wide, bool pair = false);
-int flow_whole_max_n();   // largest front the flow kernel runs as a one-warp whole-front task
-int flow_cta_max_n();     // largest front it runs as one whole-front task of a CTA
+template <typename T> void launch_sweep_flow(const SolveLaunch& a, int sweep, const FlowQueue& q, const FlowShape& sh,
+                                             int grid, const void* in, void* out, cudaStream_t s);
+int flow_blocks_per_sm(int elem_bytes, const FlowShape& sh);
 // one bounded wait on a zero flag (gives up, sets *err); for the self-test entry point
 cudaError_t launch_wait_probe(const int* flag, int* err, cudaStream_t s);
 

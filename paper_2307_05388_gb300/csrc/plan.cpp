@@ -182,13 +182,19 @@ std::string build_plan(int nx, int ny, int bx0, int by0, int bw, int bh, int lea
     const Node& nd = B.nodes[order[f]];
     d.ldk = (int)round_up(d.k, 4);
     d.iv_off = iv;
-    iv += round_up((long long)d.k * d.ldk, 64);
+    if (d.n > kTrimMaxN) iv += round_up((long long)d.k * d.ldk, 64);   // the others' inverses are packed
     d.idx_off = io;
     for (int c : nd.piv) p.idx.push_back(c);
     for (int c : bnd[f]) p.idx.push_back(c);
     io += d.n;
-    d.st_off = st;
-    st += round_up((long long)d.n * d.ld, 64);
+    if (d.n <= kTrimMaxN) {   // the update matrix only
+      d.ld = (int)round_up(d.m, 4);
+      d.st_off = st - (long long)d.k * d.ld - d.k;
+      st += round_up((long long)d.m * d.ld, 64);
+    } else {
+      d.st_off = st;
+      st += round_up((long long)d.n * d.ld, 64);
+    }
     d.v_off = vo;
     vo += round_up(d.n, 4);
     d.piv_off = po;
@@ -289,6 +295,19 @@ std::string build_plan(int nx, int ny, int bx0, int by0, int bw, int bh, int lea
   for (const auto& d : p.fronts) p.n_levels = std::max(p.n_levels, d.level + 1);
   p.level_fronts.assign(p.n_levels, {});
   for (int f = 0; f < nn; ++f) p.level_fronts[p.fronts[f].level].push_back(f);
+  p.sweep_order.reserve(nn);
+  for (const auto& lf : p.level_fronts)
+    for (int cls = 0; cls < 3; ++cls)
+      for (int f : lf) {
+        FrontDesc& d = p.fronts[f];
+        if ((d.n <= kTrimMaxN ? 0 : d.n <= kPackMaxN ? 1 : 2) != cls) continue;
+        p.sweep_order.push_back(f);
+        d.pk_off = -1;
+        if (d.n <= kPackMaxN) {
+          d.pk_off = p.pack_total;
+          p.pack_total += pack_block(d.m, d.k);
+        }
+      }
   for (const auto& d : p.fronts) {
     double k = d.k, m = d.m;
     double cfma = k * k * k / 3.0 + k * k * m + k * m * m;   // complex multiply-adds

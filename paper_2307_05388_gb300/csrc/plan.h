@@ -38,7 +38,34 @@ struct FrontDesc {           // plain-old-data, uploaded to the device as is
   int design;                // 1 if the subtree holds a design pixel (refactored on design change)
   int ldk;                   // row stride of the k x k inverse block (k rounded up to 4)
   long long iv_off;          // element offset of the inverse block (L11^-1 strictly lower, U11^-1 upper)
+  long long pk_off;          // element offset of the packed block in each half (n <= kPackMaxN), see below
 };
+
+// Small fronts (n <= kPackMaxN) keep what the sweeps read in a packed store of two equal halves,
+// one for the L side and one for the U side, a block of pack_block(m, k) entries per front in
+// each, in sweep order, so that the blocks of neighbouring fronts are one contiguous copy:
+//   - the triangle by diagonals, pack_diag(t, k) + i the entry at distance t:
+//       L side: L11^-1[i + t][i] (t = 0: 1 / d in the symmetric form, unused in LU),
+//       U side: U11^-1[i][i + t];
+//   - L21, or U12 transposed: m rows of pack_stride(k) entries;
+//   - L side: the pivot permutation (k ints).
+// Diagonals and the odd row stride let the lanes of a warp walk rows or columns of a
+// shared-memory copy without bank conflicts.
+// Fronts of up to kTrimMaxN unknowns store nothing but their update matrix in the front store:
+// row stride ld = m rounded up to 4, st_off set back so that entry (i, j) of the front, both
+// >= k, is at st_off + i * ld + j as for the other fronts.
+constexpr int kPackMaxN = 96;
+constexpr int kTrimMaxN = 64;
+#ifdef __CUDACC__
+#define FDFD_HD __host__ __device__
+#else
+#define FDFD_HD
+#endif
+FDFD_HD inline int pack_stride(int k) { return k | 1; }
+FDFD_HD inline int pack_diag(int t, int k) { return t * k - t * (t - 1) / 2; }
+FDFD_HD inline int pack_rect(int k) { return k * (k + 1) / 2; }                       // where the rows start
+FDFD_HD inline int pack_perm(int m, int k) { return pack_rect(k) + m * (k | 1); }     // where the permutation is
+FDFD_HD inline int pack_block(int m, int k) { return (pack_perm(m, k) + (k + 1) / 2 + 1) / 2 * 2; }
 
 struct Plan {
   int nx = 0, ny = 0;
@@ -55,6 +82,8 @@ struct Plan {
   int n_levels = 0;
   std::vector<std::vector<int>> level_fronts;  // front ids per level
   long long store_total = 0;          // elements of front storage per omega
+  std::vector<int> sweep_order;       // fronts by level, within a level n <= kTrimMaxN, n <= kPackMaxN, the others
+  long long pack_total = 0;           // elements of one half of the packed store per omega
   long long inv_total = 0;            // elements of the triangular-inverse storage per omega
   long long vec_total = 0;            // elements of front vectors per RHS per omega
   int perm_total = 0;

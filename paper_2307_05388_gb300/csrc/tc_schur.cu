@@ -31,6 +31,7 @@
 // drains its copies (bounded), frees its tensor memory and returns.
 #include <cuda_bf16.h>
 
+#include "async.cuh"
 #include "kernels.h"
 
 namespace fdfd {
@@ -75,47 +76,6 @@ __device__ __forceinline__ constexpr int prod_b(int form, int i) {
   return form == 2 ? (i == 1 ? 1 : 0) : form == 3 ? (i == 0 ? 0 : i == 1 ? 2 : i == 2 ? 1 : i == 3 ? 0 : i == 4 ? 1 : 0) : 0;
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Wait for the phase with the given parity to complete; false after limit_ns of
-// global time (or 2^26 polls, should the timer not advance).
-__device__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = gtimer();
-  for (uint32_t it = 1; it < (1u << 26); ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 63) == 0 && gtimer() - t0 > limit_ns) return false;
-  }
-  return false;
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // Shared-memory matrix descriptor, canonical K-major layout without swizzle:
@@ -274,9 +234,6 @@ schur_pack_kernel(FactorLaunch a, TcLaunch t) {
 
 constexpr unsigned long long kRoleWaitNs = 2000000000ull;   // copy / MMA waits
 constexpr unsigned long long kDoneWaitNs = 6000000000ull;   // accumulation waits: outlast both roles
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 
 // One CTA per output tile (slot, mt, nt): F22[128 mt.., 128 nt..] -= (L21 U12) tile.
 // Warp 0 (lane 0) streams the plane tiles, warp 1 (lane 0) issues the MMAs, warps
@@ -321,7 +278,7 @@ schur_tc_kernel(FactorLaunch a, TcLaunch t) {
     }
     mbar_init(done, 1);
     sh[1] = 0; sh[2] = 0; sh[3] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_init_fence();
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
