@@ -163,15 +163,17 @@ struct fdfd_ctx {
   // FGMRES workspace
   int gm_nrhs = 0, gm_m = 0;
   double2 *d_V = nullptr, *d_Z = nullptr, *d_r = nullptr, *d_w = nullptr;
-  double2 *d_h = nullptr, *d_h2 = nullptr, *d_hn = nullptr, *d_bd = nullptr;
+  double2 *d_h = nullptr, *d_h2 = nullptr, *d_hn = nullptr, *d_e2 = nullptr;
   double2 *d_H = nullptr, *d_cs = nullptr, *d_sn = nullptr, *d_g = nullptr, *d_ycoef = nullptr;
   double2* d_partial = nullptr;
-  double *d_vscale = nullptr, *d_resid = nullptr, *d_bnorm = nullptr;
-  int *d_active = nullptr, *d_nj = nullptr;
-  int* d_gcnt = nullptr;           // per-system counters of the Arnoldi passes (zero between launches)
-  int* h_active = nullptr;          // pinned
-  int* h_nj = nullptr;              // pinned: Krylov vectors each system used in the last cycle
-  double* h_resid = nullptr;        // pinned
+  double *d_vscale = nullptr, *d_bnorm = nullptr, *d_loss = nullptr;
+  int *d_nj = nullptr, *d_again = nullptr;
+  int* d_gcnt = nullptr;           // per-system counters of the FGMRES passes (zero between launches)
+  // what the host reads of a solve, in one copy: [resid][active, nj_out, reorth][error word]
+  unsigned char* d_stat = nullptr;
+  unsigned char* h_stat = nullptr;  // pinned
+  size_t stat_bytes = 0;
+  bool gm_second[2] = {false, false};   // the next solve runs the second projection [transpose]
 
   // per-kernel profile (CUDA events around every launch when enabled)
   bool prof_on = false;
@@ -297,14 +299,17 @@ void free_ws(fdfd_ctx* c) {
 }
 
 void free_gm(fdfd_ctx* c) {
-  void* ps[] = {c->d_V, c->d_Z, c->d_r, c->d_w, c->d_h, c->d_h2, c->d_hn, c->d_bd, c->d_H, c->d_cs,
-                c->d_sn, c->d_g, c->d_ycoef, c->d_partial, c->d_vscale, c->d_resid, c->d_bnorm,
-                c->d_active, c->d_nj, c->d_gcnt};
+  void* ps[] = {c->d_V, c->d_Z, c->d_r, c->d_w, c->d_h, c->d_h2, c->d_hn, c->d_e2, c->d_H, c->d_cs,
+                c->d_sn, c->d_g, c->d_ycoef, c->d_partial, c->d_vscale, c->d_bnorm, c->d_loss,
+                c->d_nj, c->d_again, c->d_gcnt, c->d_stat};
   for (void* p : ps) free_ptr(p);
-  c->d_V = c->d_Z = c->d_r = c->d_w = c->d_h = c->d_h2 = c->d_hn = c->d_bd = nullptr;
+  c->d_V = c->d_Z = c->d_r = c->d_w = c->d_h = c->d_h2 = c->d_hn = c->d_e2 = nullptr;
   c->d_H = c->d_cs = c->d_sn = c->d_g = c->d_ycoef = c->d_partial = nullptr;
-  c->d_vscale = c->d_resid = c->d_bnorm = nullptr;
-  c->d_active = c->d_nj = c->d_gcnt = nullptr;
+  c->d_vscale = c->d_bnorm = c->d_loss = nullptr;
+  c->d_nj = c->d_again = c->d_gcnt = nullptr;
+  c->d_stat = nullptr;
+  if (c->h_stat) cudaFreeHost(c->h_stat);
+  c->h_stat = nullptr;
   c->gm_nrhs = c->gm_m = 0;
 }
 
@@ -818,6 +823,7 @@ DevCoef dev_coef(const fdfd_ctx* c) {
   DevCoef C;
   C.cxm = c->d_cxm; C.cxp = c->d_cxp; C.cym = c->d_cym; C.cyp = c->d_cyp;
   C.k0dx2 = c->d_k0dx2; C.eps = c->d_eps; C.nx = c->nx; C.ny = c->ny;
+  C.px = c->pml.npml_x; C.py = c->pml.npml_y;
   C.sxc = c->d_sxc; C.syc = c->d_syc;
   return C;
 }
@@ -1279,39 +1285,44 @@ fdfd_status precond(fdfd_ctx* ctx, int nrhs, int transpose, const double2* src, 
   return sweeps<float2>(ctx, nrhs, transpose, src, dst);
 }
 
+// Partial sums of an FGMRES pass for up to nrhs right-hand sides per wavelength (fewer systems may
+// split into more chunks).
+long long max_partials(const fdfd_ctx* ctx, int nrhs) {
+  long long most = 1;
+  for (int r = 1; r <= nrhs; ++r) most = std::max(most, arnoldi_partials(n_cells(ctx), ctx->n_omega * r));
+  return most;
+}
+
 fdfd_status ensure_gm(fdfd_ctx* ctx, int nrhs, int m) {
   if (ctx->gm_nrhs >= nrhs && ctx->gm_m >= m) return FDFD_OK;
   free_gm(ctx);
   const size_t S = (size_t)ctx->n_omega * nrhs;
   const size_t N = (size_t)n_cells(ctx);
   const int D = multidot_max_vectors();
-  const int nblk = multidot_blocks((long long)N);
   CK(dalloc(&ctx->d_V, sizeof(double2) * (m + 1) * S * N));
   CK(dalloc(&ctx->d_Z, sizeof(double2) * m * S * N));
   CK(dalloc(&ctx->d_r, sizeof(double2) * S * N));
   CK(dalloc(&ctx->d_w, sizeof(double2) * S * N));
   CK(dalloc(&ctx->d_h, sizeof(double2) * S * D));
   CK(dalloc(&ctx->d_h2, sizeof(double2) * S * D));
-  CK(dalloc(&ctx->d_hn, sizeof(double2) * S * D));
-  CK(dalloc(&ctx->d_bd, sizeof(double2) * S * D));
+  CK(dalloc(&ctx->d_hn, sizeof(double2) * S));
+  CK(dalloc(&ctx->d_e2, sizeof(double2) * S));
   CK(dalloc(&ctx->d_H, sizeof(double2) * S * m * (m + 1)));
   CK(dalloc(&ctx->d_cs, sizeof(double2) * S * m));
   CK(dalloc(&ctx->d_sn, sizeof(double2) * S * m));
   CK(dalloc(&ctx->d_g, sizeof(double2) * S * (m + 1)));
   CK(dalloc(&ctx->d_ycoef, sizeof(double2) * S * D));
-  CK(dalloc(&ctx->d_partial, sizeof(double2) * S * D * std::max(nblk, arnoldi_blocks((long long)N))));
+  CK(dalloc(&ctx->d_partial, sizeof(double2) * (size_t)max_partials(ctx, nrhs)));
   CK(dalloc(&ctx->d_vscale, sizeof(double) * S));
-  CK(dalloc(&ctx->d_resid, sizeof(double) * S));
   CK(dalloc(&ctx->d_bnorm, sizeof(double) * S));
-  CK(dalloc(&ctx->d_active, sizeof(int) * S));
+  CK(dalloc(&ctx->d_loss, sizeof(double) * S));
   CK(dalloc(&ctx->d_nj, sizeof(int) * S));
+  CK(dalloc(&ctx->d_again, sizeof(int) * S));
   CK(dalloc(&ctx->d_gcnt, sizeof(int) * S));
   CK(cudaMemsetAsync(ctx->d_gcnt, 0, sizeof(int) * S, ctx->stream));
-  if (!ctx->h_active) {
-    CK(cudaMallocHost((void**)&ctx->h_active, sizeof(int) * 4096));
-    CK(cudaMallocHost((void**)&ctx->h_nj, sizeof(int) * 4096));
-    CK(cudaMallocHost((void**)&ctx->h_resid, sizeof(double) * 4096));
-  }
+  ctx->stat_bytes = (sizeof(double) + 3 * sizeof(int)) * S + sizeof(int);
+  CK(dalloc(&ctx->d_stat, ctx->stat_bytes));
+  CK(cudaMallocHost((void**)&ctx->h_stat, ctx->stat_bytes));
   ctx->gm_nrhs = nrhs;
   ctx->gm_m = m;
   return FDFD_OK;
@@ -1328,19 +1339,37 @@ fdfd_status check_flow_err(fdfd_ctx* ctx) {
                                                 : "a sweep gave up waiting for a front it depends on");
 }
 
-fdfd_status any_active(fdfd_ctx* ctx, int S, bool* any, double* maxres) {
-  CK(cudaMemcpyAsync(ctx->h_active, ctx->d_active, sizeof(int) * S, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->h_nj, ctx->d_nj, sizeof(int) * S, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->h_resid, ctx->d_resid, sizeof(double) * S, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->h_flow_err, ctx->d_flow_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+// Views of the status block for S systems (device or pinned).
+struct GmStat {
+  double* resid;
+  int *active, *nj_out, *reorth, *err;
+};
+GmStat gm_stat(unsigned char* p, int S) {
+  GmStat g;
+  g.resid = reinterpret_cast<double*>(p);
+  g.active = reinterpret_cast<int*>(g.resid + S);
+  g.nj_out = g.active + S;
+  g.reorth = g.nj_out + S;
+  g.err = g.reorth + S;
+  return g;
+}
+
+// Reads the status block (the pass that starts a cycle left the sweeps' error word in it; inside a
+// cycle `inside` fetches that too).
+fdfd_status any_active(fdfd_ctx* ctx, int S, bool inside, bool* any, double* maxres) {
+  const GmStat h = gm_stat(ctx->h_stat, S), d = gm_stat(ctx->d_stat, S);
+  if (inside) CK(cudaMemcpyAsync(d.err, ctx->d_flow_err, sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
+  CK(cudaMemcpyAsync(ctx->h_stat, ctx->d_stat, (sizeof(double) + 3 * sizeof(int)) * S + sizeof(int),
+                     cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
+  *ctx->h_flow_err = *h.err;
   if (ctx->growth_pending) ctx->growth_ready = true;
   CKS(check_flow_err(ctx));
   *any = false;
   *maxres = 0;
   for (int i = 0; i < S; ++i) {
-    if (ctx->h_active[i]) *any = true;
-    const double r = ctx->h_resid[i];
+    if (h.active[i]) *any = true;
+    const double r = h.resid[i];
     if (!(r <= *maxres)) *maxres = r;
   }
   return FDFD_OK;
@@ -1354,15 +1383,21 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
   if (S > 4096) return fail(ctx, FDFD_ERR_ARG, "too many systems for one solve (max 4096)");
   const long long N = n_cells(ctx);
   const size_t vs = (size_t)S * N;   // stride between Krylov vectors
-  const int D = multidot_max_vectors();
-  const int nblk = multidot_blocks(N);
   const double tol = ctx->opt.ir_tol;
-  const DevCoef C = dev_coef(ctx);
+  const int tr = transpose ? 1 : 0;
   cudaStream_t s = ctx->stream;
-  CK(cudaMemsetAsync(x, 0, sizeof(double2) * vs, s));
-  CK(cudaMemcpyAsync(ctx->d_r, b, sizeof(double2) * vs, cudaMemcpyDeviceToDevice, s));
-  { Prof pr(ctx, PK_DOT, 8.0 * N * S, 16.0 * N * S);
-    launch_multidot(b, 0, 1, b, N, S, ctx->d_partial, nblk, ctx->d_bd, D, s); }
+  const GmStat ds = gm_stat(ctx->d_stat, S), hs = gm_stat(ctx->h_stat, S);
+  ArnoldiStep as;
+  as.C = dev_coef(ctx); as.nrhs = nrhs; as.transpose = transpose;
+  as.b = b; as.z = x; as.V = ctx->d_V; as.vstride = (long long)vs; as.nv = 0; as.w = ctx->d_r;
+  as.partial = ctx->d_partial; as.cnt = ctx->d_gcnt;
+  as.h1 = ctx->d_h; as.h2 = ctx->d_h2; as.e2 = ctx->d_e2; as.hn = ctx->d_hn;
+  as.nj = ctx->d_nj; as.nj_out = ds.nj_out; as.active = ds.active; as.resid = ds.resid; as.bnorm = ctx->d_bnorm;
+  as.vscale = ctx->d_vscale; as.H = ctx->d_H; as.cs = ctx->d_cs; as.sn = ctx->d_sn; as.g = ctx->d_g;
+  as.loss = ctx->d_loss; as.reorth = ds.reorth; as.again = ctx->d_again; as.second = ctx->gm_second[tr] ? 1 : 0;
+  as.m = m; as.tol = tol; as.err = ctx->d_flow_err; as.err_out = ds.err;
+  { Prof pr(ctx, PK_DOT, 4.0 * N * S, 16.0 * N * S); launch_arnoldi(as, S, kPassStart, s); }
+  CK(cudaGetLastError());
   long long total = 0;
   double res = 0;
   bool converged = false;
@@ -1370,44 +1405,38 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
   for (int cycle = 0;; ++cycle) {
     cycles = cycle;
     if (cycle > 0) {
-      Prof pr(ctx, PK_STENCIL, 48.0 * N * S, 56.0 * N * S);
-      launch_stencil(C, ctx->n_omega, nrhs, transpose, x, b, ctx->d_r, 1, s);
+      as.z = x; as.nv = 0; as.w = ctx->d_r;
+      Prof pr(ctx, PK_STENCIL, 52.0 * N * S, 56.0 * N * S);
+      launch_arnoldi(as, S, kPassResid, s);
     }
-    { Prof pr(ctx, PK_DOT, 8.0 * N * S, 16.0 * N * S);
-      launch_multidot(ctx->d_r, 0, 1, ctx->d_r, N, S, ctx->d_partial, nblk, ctx->d_hn, D, s); }
-    { Prof pr(ctx, PK_OTHER, 0, 0);
-    gm_start(ctx->d_hn, D, ctx->d_bd, D, S, tol, m, ctx->d_g, ctx->d_vscale, ctx->d_active, ctx->d_resid,
-             ctx->d_bnorm, cycle == 0 ? 1 : 0, s); }
     CK(cudaGetLastError());
     bool any = true;
     // The first cycle starts from x = 0 (r = b), so nothing can have converged
     // yet; later cycles start from the true FP64 residual and decide.
-    if (cycle > 0 || ctx->opt.ir_max_iter == 0) {
-      CKS(any_active(ctx, S, &any, &res));
+    if (cycle > 0) {
+      CKS(any_active(ctx, S, false, &any, &res));
       if (!any) { converged = res <= tol; break; }   // a NaN residual is never converged
     }
-    if (total >= ctx->opt.ir_max_iter) break;
-    { Prof pr(ctx, PK_OTHER, 0, 32.0 * N * S); gm_scale(ctx->d_V, ctx->d_r, ctx->d_vscale, N, S, s); }
-    CK(cudaMemsetAsync(ctx->d_nj, 0, sizeof(int) * S, s));
+    if (total >= ctx->opt.ir_max_iter) {
+      if (cycle == 0) CK(cudaMemsetAsync(x, 0, sizeof(double2) * vs, s));
+      break;
+    }
+    { Prof pr(ctx, PK_OTHER, 0, 32.0 * N * S); gm_scale(ctx->d_V, cycle > 0 ? ctx->d_r : b, ctx->d_vscale, N, S, s); }
     int jdone = 0;
     for (int j = 0; j < m; ++j) {
       double2* Vj = ctx->d_V + (size_t)j * vs;
       double2* Zj = ctx->d_Z + (size_t)j * vs;
       CKS(precond(ctx, nrhs, transpose, Vj, Zj));
-      // w = A z_j, classical Gram-Schmidt applied twice, |w|, Givens update: three passes
-      ArnoldiStep as;
-      as.C = C; as.nrhs = nrhs; as.transpose = transpose;
-      as.z = Zj; as.V = ctx->d_V; as.vstride = (long long)vs; as.nv = j + 1; as.w = ctx->d_w;
-      as.partial = ctx->d_partial; as.cnt = ctx->d_gcnt;
-      as.h1 = ctx->d_h; as.h2 = ctx->d_h2; as.hn = ctx->d_hn;
-      as.nj = ctx->d_nj; as.active = ctx->d_active; as.resid = ctx->d_resid; as.bnorm = ctx->d_bnorm;
-      as.vscale = ctx->d_vscale; as.H = ctx->d_H; as.cs = ctx->d_cs; as.sn = ctx->d_sn; as.g = ctx->d_g;
-      as.m = m; as.tol = tol;
+      // e = A z_j - v_j, its projection, |e|, Givens update
+      as.z = Zj; as.nv = j + 1; as.w = ctx->d_w;
       const double pf = 8.0 * (j + 1) * N * S, pb = 16.0 * (j + 3) * N * S;
-      { Prof pr(ctx, PK_ARNOLDI, 48.0 * N * S + pf, 40.0 * N * S + 16.0 * (j + 1) * N * S);
-        launch_arnoldi(as, S, 0, s); }
-      { Prof pr(ctx, PK_ARNOLDI, 2.0 * pf, pb); launch_arnoldi(as, S, 1, s); }
-      { Prof pr(ctx, PK_ARNOLDI, pf + 4.0 * N * S, pb); launch_arnoldi(as, S, 2, s); }
+      { Prof pr(ctx, PK_ARNOLDI, 54.0 * N * S + pf, 40.0 * N * S + 16.0 * (j + 1) * N * S);
+        launch_arnoldi(as, S, kPassApply, s); }
+      { Prof pr(ctx, PK_ARNOLDI, pf + 4.0 * N * S, pb); launch_arnoldi(as, S, kPassProj, s); }
+      if (as.second) {
+        { Prof pr(ctx, PK_ARNOLDI, 0, 0); launch_arnoldi(as, S, kPassDots2, s); }
+        { Prof pr(ctx, PK_ARNOLDI, 0, 0); launch_arnoldi(as, S, kPassProj2, s); }
+      }
       CK(cudaGetLastError());
       ++total;
       jdone = j + 1;
@@ -1417,9 +1446,9 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
       // the expectation holds; a restart when it does not).  Later cycles look at
       // the convergence flags after every iteration; meanwhile the device-side
       // flags already freeze converged systems (zero search directions, no updates).
-      if (cycle == 0 && total == ctx->gm_expect[transpose ? 1 : 0] && total < ctx->opt.ir_max_iter) break;
-      if (total >= ctx->gm_expect[transpose ? 1 : 0] || j + 1 == m || total >= ctx->opt.ir_max_iter) {
-        CKS(any_active(ctx, S, &any, &res));
+      if (cycle == 0 && total == ctx->gm_expect[tr] && total < ctx->opt.ir_max_iter) break;
+      if (total >= ctx->gm_expect[tr] || j + 1 == m || total >= ctx->opt.ir_max_iter) {
+        CKS(any_active(ctx, S, true, &any, &res));
         if (!any) break;
       }
       if (total >= ctx->opt.ir_max_iter) break;
@@ -1430,7 +1459,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
     }
     { Prof pr(ctx, PK_OTHER, 0, 0); gm_solve(ctx->d_H, ctx->d_g, S, m, ctx->d_nj, ctx->d_ycoef, s); }
     { Prof pr(ctx, PK_AXPY, 8.0 * jdone * N * S, 16.0 * (jdone + 2) * N * S);
-      launch_multiaxpy(ctx->d_Z, (long long)vs, jdone, ctx->d_ycoef, D, x, N, S, nullptr, s); }
+      launch_multiaxpy(ctx->d_Z, (long long)vs, jdone, ctx->d_ycoef, multidot_max_vectors(), x, N, S, cycle == 0, s); }
     CK(cudaGetLastError());
   }
   ctx->last_iters = total;
@@ -1442,10 +1471,15 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
   long long expect = total;
   if (converged && cycles == 1) {
     int mx = 0;
-    for (int i = 0; i < S; ++i) mx = std::max(mx, ctx->h_nj[i]);
+    for (int i = 0; i < S; ++i) mx = std::max(mx, hs.nj_out[i]);
     if (mx > 0) expect = std::min<long long>(expect, mx);
   }
-  ctx->gm_expect[transpose ? 1 : 0] = std::max<long long>(1, expect);
+  ctx->gm_expect[tr] = std::max<long long>(1, expect);
+  // the second projection runs in the next solve if a system of this one wanted it
+  if (cycles > 0) {
+    ctx->gm_second[tr] = false;
+    for (int i = 0; i < S; ++i) ctx->gm_second[tr] = ctx->gm_second[tr] || hs.reorth[i] != 0;
+  }
   if (!converged)
     return fail(ctx, FDFD_ERR_NOT_CONVERGED,
                 "refinement stopped at relative residual " + std::to_string(res) + " after " +
@@ -2251,9 +2285,6 @@ void fdfd_destroy(fdfd_ctx* ctx) {
   }
   if (ctx->h_growth_max) cudaFreeHost(ctx->h_growth_max);
   if (ctx->h_flow_err) cudaFreeHost(ctx->h_flow_err);
-  if (ctx->h_active) cudaFreeHost(ctx->h_active);
-  if (ctx->h_nj) cudaFreeHost(ctx->h_nj);
-  if (ctx->h_resid) cudaFreeHost(ctx->h_resid);
   delete ctx;
 }
 

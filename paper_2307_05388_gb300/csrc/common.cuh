@@ -97,6 +97,7 @@ struct DevCoef {
   const double2* sxc;    // [n_omega][nx]  stretch s_x at cell centres
   const double2* syc;    // [n_omega][ny]  stretch s_y at cell centres
   int nx, ny;
+  int px, py;            // PML cells on each side of an axis: the couplings are -1 between them
 };
 
 // D[cell] = s_x(i + 1/2) s_y(j + 1/2): the diagonal for which D A is complex

@@ -200,50 +200,47 @@ cudaError_t launch_wait_probe(const int* flag, int* err, cudaStream_t s);
 // y = A x (op = 0) or r = b - A x (op = 1), FP64 matrix-free stencil, all systems.
 void launch_stencil(const DevCoef& c, int n_omega, int nrhs, int transpose, const double2* x,
                     const double2* b, double2* y, int op, cudaStream_t s);
-// batched dot products h[s][i] = sum conj(V_i[s]) w[s], i < nv (V_i at V + i*vstride)
-void launch_multidot(const double2* V, long long vstride, int nv, const double2* w, long long n,
-                     int nsys, double2* partial, int nblk, double2* out, int out_ld, cudaStream_t s);
-// w[s] -= sum_i h[s][i] V_i[s]
+// w[s] -= sum_i h[s][i] V_i[s], or with set w[s] = -sum_i h[s][i] V_i[s]
 void launch_multiaxpy(const double2* V, long long vstride, int nv, const double2* h, int h_ld,
-                      double2* w, long long n, int nsys, const int* active, cudaStream_t s);
-int multidot_blocks(long long n);
+                      double2* w, long long n, int nsys, int set, cudaStream_t s);
 int multidot_max_vectors();
-int arnoldi_blocks(long long n);   // chunks of an Arnoldi pass (partial sums per output)
 
-// FGMRES bookkeeping (one thread per system); see vec.cu
-void gm_start(const double2* rr, int rr_ld, const double2* bb, int bb_ld, int nsys, double tol, int m,
-              double2* g, double* vscale, int* active, double* resid, double* bnorm, int first, cudaStream_t s);
 void gm_solve(const double2* H, const double2* g, int nsys, int m, const int* njs, double2* ny_out,
               cudaStream_t s);
 void gm_scale(double2* dst, const double2* src, const double* scale, long long n, int nsys, cudaStream_t s);
-// One FGMRES Arnoldi step (classical Gram-Schmidt twice, then the Givens
-// update) for every active system in three launches, pass = 0, 1, 2:
-//   0: w = A z (A^T if transpose), h1 = V^H w;  1: w -= V h1, h2 = V^H w;
-//   2: w -= V h2, hn = |w|^2, column nv - 1 of H from h1 + h2 and hn, nj += 1.
-// h1, h2, hn: [nsys][multidot_max_vectors()]; partial: [nsys][multidot_max_vectors()]
-// [arnoldi_blocks(n)];
-// cnt: [nsys] zero, left zero.
+// One pass of FGMRES for every system (for every active one inside a cycle); see vec.cu.
+enum ArnoldiPass { kPassStart = 0, kPassResid, kPassApply, kPassProj, kPassDots2, kPassProj2 };
 struct ArnoldiStep {
   DevCoef C;
   int nrhs, transpose;
-  const double2* z;
+  const double2* b;        // right-hand sides (kPassStart, kPassResid)
+  const double2* z;        // what A is applied to: x (kPassResid), z_j (kPassApply)
   const double2* V;
   long long vstride;
   int nv;                  // V_0 .. V_{nv-1}; the step is j = nv - 1
-  double2* w;
-  double2* partial;
-  int* cnt;
-  double2 *h1, *h2, *hn;
-  int* nj;
+  double2* w;              // the pass's vector: r, or the next Krylov vector
+  double2* partial;        // [arnoldi_partials(n, nsys)]
+  int* cnt;                // [nsys] zero, left zero
+  double2 *h1, *h2;        // projections, [nsys][multidot_max_vectors()]
+  double2 *e2, *hn;        // squared norms (x), [nsys]
+  int* nj;                 // Krylov vectors used in this cycle, [nsys]
+  int* nj_out;             // ... in the one before, [nsys]
   int* active;
   double* resid;
-  const double* bnorm;
+  double* bnorm;
   double* vscale;
   double2 *H, *cs, *sn, *g;
+  double* loss;            // orthogonality lost so far, [nsys]
+  int* reorth;             // 1: this solve needed (or wanted) a second projection, [nsys]
+  int* again;              // 1: kPassProj left the column to the second projection, [nsys]
+  int second;              // the second projection's passes are launched
   int m;
   double tol;
+  const int* err;          // the sweeps' error word, copied beside the results by the passes that start a cycle
+  int* err_out;
 };
 void launch_arnoldi(const ArnoldiStep& g, int nsys, int pass, cudaStream_t s);
+long long arnoldi_partials(long long n, int nsys);
 
 // objective o = g^T x on a monitor column, F = sum weight |o|^2 with adjoint source weight conj(o) g,
 // or with target != NULL F = sum weight (|o|^2 - target)^2 with adjoint source 2 weight (|o|^2 - target) conj(o) g

@@ -65,6 +65,14 @@ __device__ __forceinline__ double2 stencil_at(const DevCoef& c, int w, int trans
                                               long long cell) {
   const int ci = (int)cell;                    // grids stay below 2^31 cells
   const int i = ci / c.ny, j = ci - i * c.ny;
+  if (i > c.px && i < c.nx - 1 - c.px && j > c.py && j < c.ny - 1 - c.py) {
+    // between the absorbing layers every coupling is exactly -1 (and A = A^T there): 9 FP64
+    // operations per cell instead of 27
+    const double2 xw = X[cell - c.ny], xe = X[cell + c.ny], xs = X[cell - 1], xn = X[cell + 1], x0 = X[cell];
+    const double dg = fma(-c.k0dx2[w], c.eps[cell], 4.0);
+    const double sx = (xw.x + xe.x) + (xs.x + xn.x), sy = (xw.y + xe.y) + (xs.y + xn.y);
+    return make_double2(fma(dg, x0.x, -sx), fma(dg, x0.y, -sy));
+  }
   const double2* cxm = c.cxm + (size_t)w * c.nx;
   const double2* cxp = c.cxp + (size_t)w * c.nx;
   const double2* cym = c.cym + (size_t)w * c.ny;
@@ -105,75 +113,15 @@ __global__ void stencil_kernel(DevCoef c, int nrhs, int transpose, const double2
 constexpr int kDotThreads = 256;
 constexpr int kMaxDot = 17;
 
-// Partial sums of h[s][i] = sum_t conj(V_i[s][t]) w[s][t]: one CTA per
-// (chunk of kDotPer * 256 entries, vector i, system), one accumulator per
-// thread (low register use keeps the FP64 pipes fed by many warps), CTA
-// reduction in a fixed order.
-constexpr int kDotPer = 4;
-constexpr int kArnPer = 2;   // entries per thread of an Arnoldi pass: FP64 FMA is 2 per SM per clock, so
-                             // the CTAs cover every SM while the FP64 adds of the reductions stay few
-
-__global__ void __launch_bounds__(kDotThreads)
-multidot_partial_kernel(const double2* __restrict__ V, long long vstride, int nv,
-                        const double2* __restrict__ w, long long n, double2* partial, int nblk) {
-  __shared__ double2 red[kDotThreads / 32];
-  const int i = blockIdx.y, sys = blockIdx.z;
-  const double2* W = w + (size_t)sys * n;
-  const double2* Vi = V + (size_t)i * vstride + (size_t)sys * n;
-  const long long t0 = (long long)blockIdx.x * (kDotThreads * kDotPer) + threadIdx.x;
-  double2 vv[kDotPer], ww[kDotPer];
-#pragma unroll
-  for (int u = 0; u < kDotPer; ++u) {
-    const long long t = t0 + (long long)u * kDotThreads;
-    vv[u] = t < n ? Vi[t] : make_double2(0, 0);
-    ww[u] = t < n ? W[t] : make_double2(0, 0);
-  }
-  double2 acc = make_double2(0, 0);
-#pragma unroll
-  for (int u = 0; u < kDotPer; ++u) acc = cfma(cconj(vv[u]), ww[u], acc);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-  }
-  if (lane == 0) red[warp] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 s = red[0];
-    for (int q = 1; q < kDotThreads / 32; ++q) s = cadd(s, red[q]);
-    partial[((size_t)sys * kMaxDot + i) * nblk + blockIdx.x] = s;
-  }
-}
-
-// One warp per (system, vector): lane-strided partial sums, then a shuffle tree
-// (fixed order, so the result does not depend on timing).
-__global__ void multidot_final_kernel(const double2* partial, int nblk, int nv, double2* out, int out_ld) {
-  const int sys = blockIdx.x;
-  const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (i >= nv) return;
-  double2 s = make_double2(0, 0);
-  const double2* p = partial + ((size_t)sys * kMaxDot + i) * nblk;
-  for (int b = lane; b < nblk; b += 32) s = cadd(s, p[b]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-  }
-  if (lane == 0) out[(size_t)sys * out_ld + i] = s;
-}
-
-// w[s] -= sum_i h[s][i] V_i[s]; the coefficients sit in shared memory.
+// w[s] -= sum_i h[s][i] V_i[s] (set: from w = 0); the coefficients sit in shared memory.
 __global__ void multiaxpy_kernel(const double2* __restrict__ V, long long vstride, int nv,
-                                 const double2* __restrict__ h, int h_ld, double2* w, long long n,
-                                 const int* active) {
+                                 const double2* __restrict__ h, int h_ld, double2* w, long long n, int set) {
   __shared__ double2 hh[kMaxDot];
   const int sys = blockIdx.y;
-  if (active && !active[sys]) return;
   if (threadIdx.x < nv) hh[threadIdx.x] = h[(size_t)sys * h_ld + threadIdx.x];
   __syncthreads();
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    double2 acc = w[(size_t)sys * n + t];
+    double2 acc = set ? make_double2(0, 0) : w[(size_t)sys * n + t];
     for (int i = 0; i < nv; ++i) acc = cfms(hh[i], V[(size_t)i * vstride + (size_t)sys * n + t], acc);
     w[(size_t)sys * n + t] = acc;
   }
@@ -208,24 +156,11 @@ void launch_stencil(const DevCoef& c, int n_omega, int nrhs, int transpose, cons
 }
 
 
-// chunks of kDotPer entries per thread
-int multidot_blocks(long long n) {
-  long long b = (n + kDotThreads * kDotPer - 1) / (kDotThreads * kDotPer);
-  if (b < 1) b = 1;
-  return (int)b;
-}
 int multidot_max_vectors() { return kMaxDot; }
-int arnoldi_blocks(long long n) { return (int)((n + kDotThreads * kArnPer - 1) / (kDotThreads * kArnPer)); }
-
-void launch_multidot(const double2* V, long long vstride, int nv, const double2* w, long long n, int nsys,
-                     double2* partial, int nblk, double2* out, int out_ld, cudaStream_t s) {
-  multidot_partial_kernel<<<dim3(nblk, nv, nsys), kDotThreads, 0, s>>>(V, vstride, nv, w, n, partial, nblk);
-  multidot_final_kernel<<<nsys, 32 * kMaxDot, 0, s>>>(partial, nblk, nv, out, out_ld);
-}
 
 void launch_multiaxpy(const double2* V, long long vstride, int nv, const double2* h, int h_ld, double2* w,
-                      long long n, int nsys, const int* active, cudaStream_t s) {
-  multiaxpy_kernel<<<dim3(grid_for(n), nsys), 256, 0, s>>>(V, vstride, nv, h, h_ld, w, n, active);
+                      long long n, int nsys, int set, cudaStream_t s) {
+  multiaxpy_kernel<<<dim3(grid_for(n), nsys), 256, 0, s>>>(V, vstride, nv, h, h_ld, w, n, set);
 }
 
 // ---------------------------------------------------------------------------
@@ -233,23 +168,23 @@ void launch_multiaxpy(const double2* V, long long vstride, int nv, const double2
 // ---------------------------------------------------------------------------
 namespace {
 
-__global__ void gm_start_kernel(const double2* rr, int rr_ld, const double2* bb, int bb_ld, int nsys,
-                                double tol, int m, double2* g, double* vscale, int* active, double* resid,
-                                double* bnorm, int first) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsys) return;
+// Start of a cycle for system s from |r|^2 (first: x = 0, r = b, and |b| is taken from it).
+__device__ void start_system(const ArnoldiStep& g, int s, double rr2, int first) {
   // norms from sums of squares; a NaN stays NaN (fmax would turn it into 0, and a
   // poisoned solve would then look converged)
-  const double rr2 = rr[(size_t)s * rr_ld].x, bb2 = bb[(size_t)s * bb_ld].x;
   const double beta = rr2 > 0.0 ? sqrt(rr2) : (rr2 == rr2 ? 0.0 : rr2);
-  if (first) bnorm[s] = bb2 > 0.0 ? sqrt(bb2) : (bb2 == bb2 ? 0.0 : bb2);
-  const double bn = bnorm[s];
-  for (int i = 0; i <= m; ++i) g[(size_t)s * (m + 1) + i] = make_double2(0, 0);
-  g[(size_t)s * (m + 1)] = make_double2(beta, 0);
-  resid[s] = bn > 0 ? beta / bn : 0.0;
-  const int act = (bn > 0) && (beta > tol * bn) && (beta == beta);
-  active[s] = act;
-  vscale[s] = act ? 1.0 / beta : 0.0;
+  if (first) g.bnorm[s] = beta;
+  const double bn = first ? beta : g.bnorm[s];
+  for (int i = 0; i <= g.m; ++i) g.g[(size_t)s * (g.m + 1) + i] = make_double2(0, 0);
+  g.g[(size_t)s * (g.m + 1)] = make_double2(beta, 0);
+  g.resid[s] = bn > 0 ? beta / bn : 0.0;
+  const int act = (bn > 0) && (beta > g.tol * bn) && (beta == beta);
+  g.active[s] = act;
+  g.vscale[s] = act ? 1.0 / beta : 0.0;
+  g.nj_out[s] = first ? 0 : g.nj[s];   // Krylov vectors of the cycle that ended
+  g.nj[s] = 0;
+  if (first) g.reorth[s] = 0;
+  g.loss[s] = 0.0;
 }
 
 // Column j of the Hessenberg matrix of system s from its projections h[0..j]
@@ -257,7 +192,8 @@ __global__ void gm_start_kernel(const double2* rr, int rr_ld, const double2* bb,
 // estimate updated; a system whose estimate meets tol (or breaks down: exact
 // solution) becomes inactive.
 __device__ void givens_step(int s, const double2* hs, double hn2, int j, int m, double tol, double2* H, double2* cs,
-                            double2* sn, double2* g, double* vscale, int* active, double* resid, const double* bnorm) {
+                            double2* sn, double2* g, double* vscale, int* active, double* resid,
+                            const double* bnorm) {
   double2* Hc = H + ((size_t)s * m + j) * (m + 1);   // column j of H
   for (int i = 0; i <= j; ++i) Hc[i] = hs[i];
   const double hnorm = hn2 > 0.0 ? sqrt(hn2) : (hn2 == hn2 ? 0.0 : hn2);
@@ -327,73 +263,144 @@ __global__ void scale_vec_kernel(double2* dst, const double2* src, const double*
 }
 
 
-// One Arnoldi step of FGMRES with classical Gram-Schmidt applied twice, for
-// every active system, in three passes over the vectors (pass p):
-//   0: w = A z_j,             h1_i = V_i^H w
-//   1: w -= sum_i h1_i V_i,   h2_i = V_i^H w
-//   2: w -= sum_i h2_i V_i,   |w|^2, then h = h1 + h2 and the Givens update
-// (the second projection is always needed here: with a preconditioner this
-// close to A^-1, A z_j lies almost in the span of V and the first projection
-// cancels most of w).
-// CTA (chunk of kArnPer * 256 entries, system); each CTA writes its partial
-// sums, and the last CTA of a system (a counter it resets afterwards) adds
-// them in chunk order, so results do not depend on timing.
-__global__ void __launch_bounds__(kDotThreads)
+// ---------------------------------------------------------------------------
+// FGMRES over the vectors of every system: one launch per pass, CTA (chunk of PER * 256 entries,
+// system).  Each CTA writes its partial sums and the last CTA of a system (a counter it resets
+// afterwards) adds them in chunk order, so results do not depend on timing, and runs the
+// system's bookkeeping.
+//
+//   kPassStart  |b|^2, start of the first cycle (x = 0)
+//   kPassResid  r = b - A x, |r|^2, start of a later cycle
+//   kPassApply  e = A z_j - v_j,             h_i = V_i^H e,  |e|^2
+//   kPassProj   e -= sum_i h_i V_i,          |e|^2, then the Givens update of column j
+//   kPassDots2  h2_i = V_i^H e               (systems marked by kPassProj)
+//   kPassProj2  e -= sum_i h2_i V_i,         |e|^2, then their Givens update
+//
+// The preconditioner is close to A^-1, so A z_j lies almost along v_j and projecting it once leaves a
+// vector that is orthogonal only to the rounding of the large component: Gram-Schmidt used to run
+// twice for that.  Taking v_j off first (h_jj = 1 + V_j^H e) removes the large component exactly, and
+// one projection of the small rest is enough unless it cancels again.  What one projection loses is
+// followed per system: loss_{j+1} = loss_j |e| / |e'| + 2^-52 / |e'|.  Where it passes 1e-3 the cycle of that
+// system ends (the next one starts from the true residual) and the host asks for the second
+// projection (kPassDots2, kPassProj2) in the next solve of that direction; it then runs where the
+// first one cancelled more than a factor of ten.
+//
+// FP64 is 2 multiply-adds per clock and SM on this part and bounds these passes.  Eight entries per thread and
+// a butterfly that halves the values with the lanes (6 additions for two complex sums where a plain
+// shuffle tree takes 20) keep the reductions' share small, and the stencil takes 9 operations between the
+// absorbing layers.
+// ---------------------------------------------------------------------------
+constexpr double kMaxLoss = 1e-3;
+
+// Sums of two complex values over the warp: lanes 0, 8, 16, 24 end up with a.x, a.y, b.x, b.y.
+__device__ __forceinline__ double warp_sum2(double2 a, double2 b, int lane) {
+  const bool up16 = lane & 16, up8 = lane & 8;
+  const double k0 = up16 ? b.x : a.x, k1 = up16 ? b.y : a.y, s0 = up16 ? a.x : b.x, s1 = up16 ? a.y : b.y;
+  const double r0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 16), r1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 16);
+  double v = (up8 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, up8 ? r0 : r1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Column nv - 1 of system s from the projections h (and h2) and |e'|^2.
+__device__ void finish_column(const ArnoldiStep& g, int s, const double2* h, const double2* h2, double hn2) {
+  double2 hs[kMaxDot];
+  for (int i = 0; i < g.nv; ++i) hs[i] = h2 ? cadd(h[i], h2[i]) : h[i];
+  hs[g.nv - 1].x += 1.0;
+  g.nj[s] += 1;
+  givens_step(s, hs, hn2, g.nv - 1, g.m, g.tol, g.H, g.cs, g.sn, g.g, g.vscale, g.active, g.resid, g.bnorm);
+}
+
+template <int PER>
+__global__ void __launch_bounds__(kDotThreads, PER >= 8 ? 2 : 3)
 arnoldi_kernel(ArnoldiStep g, int pass) {
-  __shared__ double2 red[kDotThreads / 32][kMaxDot];
+  __shared__ double red[kDotThreads / 32][2 * (kMaxDot + 1)];
   __shared__ double2 hc[kMaxDot];
   __shared__ int s_last;
   const int sys = blockIdx.y;
-  if (!g.active[sys]) return;
+  const bool begin = pass == kPassStart || pass == kPassResid;
+  if (!begin && !g.active[sys]) return;
+  if ((pass == kPassDots2 || pass == kPassProj2) && !g.again[sys]) return;
   const int nv = g.nv, nblk = gridDim.x;
   const long long n = (long long)g.C.nx * g.C.ny;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (pass > 0 && tid < nv) hc[tid] = (pass == 1 ? g.h1 : g.h2)[(size_t)sys * kMaxDot + tid];
+  const bool project = pass == kPassProj || pass == kPassProj2;
+  if (project && tid < nv) hc[tid] = (pass == kPassProj ? g.h1 : g.h2)[(size_t)sys * kMaxDot + tid];
   __syncthreads();
   double2* W = g.w + (size_t)sys * n;
   const double2* Vs = g.V + (size_t)sys * n;
-  const long long t0 = (long long)blockIdx.x * (kDotThreads * kArnPer) + tid;
-  double2 wv[kArnPer];
+  const long long t0 = (long long)blockIdx.x * (kDotThreads * PER) + tid;
+  double2 wv[PER];
 #pragma unroll
-  for (int u = 0; u < kArnPer; ++u) {
+  for (int u = 0; u < PER; ++u) {
     const long long t = t0 + (long long)u * kDotThreads;
     double2 x = make_double2(0, 0);
     if (t < n) {
-      if (pass == 0) {
-        x = stencil_at(g.C, sys / g.nrhs, g.transpose, g.z + (size_t)sys * n, t);
+      if (pass == kPassStart) {
+        x = g.b[(size_t)sys * n + t];
+      } else if (pass == kPassResid) {
+        x = csub(g.b[(size_t)sys * n + t], stencil_at(g.C, sys / g.nrhs, g.transpose, g.z + (size_t)sys * n, t));
+        W[t] = x;
+      } else if (pass == kPassApply) {
+        x = csub(stencil_at(g.C, sys / g.nrhs, g.transpose, g.z + (size_t)sys * n, t),
+                 Vs[(size_t)(nv - 1) * g.vstride + t]);
+        W[t] = x;
       } else {
         x = W[t];
-        for (int i = 0; i < nv; ++i) x = cfms(hc[i], Vs[(size_t)i * g.vstride + t], x);
       }
-      W[t] = x;
     }
     wv[u] = x;
   }
-  const int nout = pass < 2 ? nv : 1;
-  for (int i = 0; i < nout; ++i) {
-    double2 acc = make_double2(0, 0);
-    if (pass < 2) {
+  if (project) {
+    for (int i = 0; i < nv; ++i) {
+      const double2 h = hc[i];
+      const double2* Vi = Vs + (size_t)i * g.vstride;
+      double2 vv[PER];
 #pragma unroll
-      for (int u = 0; u < kArnPer; ++u) {
+      for (int u = 0; u < PER; ++u) {
         const long long t = t0 + (long long)u * kDotThreads;
-        if (t < n) acc = cfma(cconj(Vs[(size_t)i * g.vstride + t]), wv[u], acc);
+        vv[u] = t < n ? Vi[t] : make_double2(0, 0);
       }
-    } else {
 #pragma unroll
-      for (int u = 0; u < kArnPer; ++u) acc.x += wv[u].x * wv[u].x + wv[u].y * wv[u].y;
+      for (int u = 0; u < PER; ++u) wv[u] = cfms(h, vv[u], wv[u]);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    for (int u = 0; u < PER; ++u) {
+      const long long t = t0 + (long long)u * kDotThreads;
+      if (t < n) W[t] = wv[u];
     }
-    if (lane == 0) red[warp][i] = acc;
+  }
+  // outputs 0 .. nd - 1: V_i^H w; output nd: |w|^2 (but in kPassDots2)
+  const int nd = (pass == kPassApply || pass == kPassDots2) ? nv : 0;
+  const int nout = pass == kPassDots2 ? nd : nd + 1;
+  for (int i = 0; i < nout; i += 2) {
+    double2 acc[2] = {make_double2(0, 0), make_double2(0, 0)};
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      if (i + p < nd) {
+        const double2* Vi = Vs + (size_t)(i + p) * g.vstride;
+        double2 vv[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+          const long long t = t0 + (long long)u * kDotThreads;
+          vv[u] = t < n ? Vi[t] : make_double2(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < PER; ++u) acc[p] = cfma(cconj(vv[u]), wv[u], acc[p]);
+      } else if (i + p == nd) {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) acc[p].x = fma(wv[u].x, wv[u].x, fma(wv[u].y, wv[u].y, acc[p].x));
+      }
+    }
+    const double v = warp_sum2(acc[0], acc[1], lane);
+    if ((lane & 7) == 0) red[warp][2 * i + (lane >> 3)] = v;
   }
   __syncthreads();
-  if (tid < nout) {
-    double2 sum = red[0][tid];
-    for (int q = 1; q < kDotThreads / 32; ++q) sum = cadd(sum, red[q][tid]);
-    g.partial[((size_t)sys * kMaxDot + tid) * nblk + blockIdx.x] = sum;
+  if (tid < 2 * nout) {
+    double sum = red[0][tid];
+    for (int q = 1; q < kDotThreads / 32; ++q) sum += red[q][tid];
+    reinterpret_cast<double*>(g.partial)[(((size_t)sys * (kMaxDot + 1) + (tid >> 1)) * nblk + blockIdx.x) * 2 + (tid & 1)] = sum;
   }
   __threadfence();
   __syncthreads();
@@ -401,9 +408,10 @@ arnoldi_kernel(ArnoldiStep g, int pass) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  double2* out = pass == 0 ? g.h1 : (pass == 1 ? g.h2 : g.hn);
+  double2* out = pass == kPassDots2 ? g.h2 : pass == kPassApply ? g.h1 : nullptr;
+  double2* norm = (pass == kPassApply ? g.e2 : g.hn) + sys;
   for (int o = warp; o < nout; o += kDotThreads / 32) {   // warp adds outputs o, o + 8, ...: lane-strided, then a shuffle tree
-    const double2* p = g.partial + ((size_t)sys * kMaxDot + o) * nblk;
+    const double2* p = g.partial + ((size_t)sys * (kMaxDot + 1) + o) * nblk;
     double2 sum = make_double2(0, 0);
     for (int b = lane; b < nblk; b += 32) sum = cadd(sum, __ldcg(p + b));
 #pragma unroll
@@ -411,28 +419,46 @@ arnoldi_kernel(ArnoldiStep g, int pass) {
       sum.x += __shfl_xor_sync(0xffffffffu, sum.x, q);
       sum.y += __shfl_xor_sync(0xffffffffu, sum.y, q);
     }
-    if (lane == 0) out[(size_t)sys * kMaxDot + o] = sum;
+    if (lane == 0) {
+      if (o < nd) out[(size_t)sys * kMaxDot + o] = sum;
+      else *norm = sum;
+    }
   }
   if (tid == 0) g.cnt[sys] = 0;
-  if (pass == 2) {
-    __syncthreads();
-    if (tid == 0) {
-      double2 hs[kMaxDot];
-      for (int i = 0; i < nv; ++i) hs[i] = cadd(g.h1[(size_t)sys * kMaxDot + i], g.h2[(size_t)sys * kMaxDot + i]);
-      g.nj[sys] += 1;
-      givens_step(sys, hs, g.hn[(size_t)sys * kMaxDot].x, nv - 1, g.m, g.tol, g.H, g.cs, g.sn, g.g, g.vscale,
-                  g.active, g.resid, g.bnorm);
+  __syncthreads();
+  if (tid != 0) return;
+  if (begin) {
+    start_system(g, sys, norm->x, pass == kPassStart);
+    if (sys == 0) *g.err_out = *g.err;
+  } else if (project) {
+    const double2* h = g.h1 + (size_t)sys * kMaxDot;
+    const double hn2 = norm->x, en2 = g.e2[sys].x;
+    if (pass == kPassProj) {
+      const bool cancelled = hn2 < 0.01 * en2;
+      if (cancelled && g.second) {
+        g.again[sys] = 1;                 // the Givens update waits for the second projection
+        return;
+      }
+      g.again[sys] = 0;
+      finish_column(g, sys, h, nullptr, hn2);
+      const double hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
+      const double loss = hn > 0.0 ? g.loss[sys] * sqrt(en2) / hn + 2.220446049250313e-16 / hn : 0.0;
+      g.loss[sys] = loss;
+      if (loss > kMaxLoss) {
+        g.active[sys] = 0;
+        g.reorth[sys] = 1;
+      }
+    } else {
+      g.again[sys] = 0;
+      g.reorth[sys] = 1;                  // needed here: the next solve keeps the second projection
+      finish_column(g, sys, h, g.h2 + (size_t)sys * kMaxDot, hn2);
+      g.loss[sys] = 2.220446049250313e-16;
     }
   }
 }
 
 }  // namespace
 
-void gm_start(const double2* rr, int rr_ld, const double2* bb, int bb_ld, int nsys, double tol, int m,
-              double2* g, double* vscale, int* active, double* resid, double* bnorm, int first, cudaStream_t s) {
-  gm_start_kernel<<<(nsys + 63) / 64, 64, 0, s>>>(rr, rr_ld, bb, bb_ld, nsys, tol, m, g, vscale, active, resid,
-                                                  bnorm, first);
-}
 void gm_solve(const double2* H, const double2* g, int nsys, int m, const int* njs, double2* ny_out,
               cudaStream_t s) {
   gm_solve_kernel<<<(nsys + 63) / 64, 64, 0, s>>>(H, g, nsys, m, njs, ny_out);
@@ -440,9 +466,26 @@ void gm_solve(const double2* H, const double2* g, int nsys, int m, const int* nj
 void gm_scale(double2* dst, const double2* src, const double* scale, long long n, int nsys, cudaStream_t s) {
   scale_vec_kernel<<<dim3(grid_for(n), nsys), 256, 0, s>>>(dst, src, scale, n);
 }
+// Entries per thread: eight, but few enough that the CTAs still cover the SMs three times over.
+static int arnoldi_per(long long n, int nsys) {
+  int per = 8;
+  while (per > 1 && (n + kDotThreads * per - 1) / (kDotThreads * per) * nsys < 3 * 152) per /= 2;
+  return per;
+}
+long long arnoldi_partials(long long n, int nsys) {
+  const int per = arnoldi_per(n, nsys);
+  return (long long)nsys * (kMaxDot + 1) * ((n + kDotThreads * per - 1) / (kDotThreads * per));
+}
 void launch_arnoldi(const ArnoldiStep& g, int nsys, int pass, cudaStream_t s) {
   const long long n = (long long)g.C.nx * g.C.ny;
-  arnoldi_kernel<<<dim3(arnoldi_blocks(n), nsys), kDotThreads, 0, s>>>(g, pass);
+  const int per = arnoldi_per(n, nsys);
+  const dim3 grid((unsigned)((n + kDotThreads * per - 1) / (kDotThreads * per)), nsys);
+  switch (per) {
+    case 8: arnoldi_kernel<8><<<grid, kDotThreads, 0, s>>>(g, pass); break;
+    case 4: arnoldi_kernel<4><<<grid, kDotThreads, 0, s>>>(g, pass); break;
+    case 2: arnoldi_kernel<2><<<grid, kDotThreads, 0, s>>>(g, pass); break;
+    default: arnoldi_kernel<1><<<grid, kDotThreads, 0, s>>>(g, pass); break;
+  }
 }
 
 // ---------------------------------------------------------------------------
