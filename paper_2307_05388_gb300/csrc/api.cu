@@ -322,6 +322,7 @@ fdfd_status analyze_host(fdfd_ctx* ctx) {
   if (!e.empty()) return fail(ctx, FDFD_ERR_ARG, "symbolic phase: " + e);
   for (const auto& d : ctx->plan.fronts)
     if (d.nchild > 2) return fail(ctx, FDFD_ERR_ARG, "symbolic phase: front with more than two children");
+  flag_interior(&ctx->plan, ctx->pml.npml_x, ctx->pml.npml_y);
   ctx->analyzed = true;
   ctx->sf += 1;
   return FDFD_OK;

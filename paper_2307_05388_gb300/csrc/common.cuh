@@ -109,8 +109,13 @@ __device__ __forceinline__ double2 sym_scale(const DevCoef& c, int w, int cell) 
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Value of the stencil entry with code = cell*5 + direction at wavelength w.
+// Value of the stencil entry with code = cell*5 + direction (| kInterior) at wavelength w.
 __device__ __forceinline__ double2 stencil_entry(const DevCoef& c, int w, int code) {
+  if (code < 0) {   // between the absorbing layers
+    code &= ~kInterior;
+    const int at = code / 5;
+    return make_double2(code - at * 5 == DIR_DIAG ? fma(-c.k0dx2[w], c.eps[at], 4.0) : -1.0, 0.0);
+  }
   int cell = code / 5, dir = code - cell * 5;
   int i = cell / c.ny, j = cell - i * c.ny;
   const double2 xm = c.cxm[(size_t)w * c.nx + i], xp = c.cxp[(size_t)w * c.nx + i];

@@ -270,7 +270,8 @@ std::string build_plan(int nx, int ny, int bx0, int by0, int bw, int bh, int lea
         p.orig_ptr.push_back(base + (int)e);
       }
       for (auto& en : ent) {
-        p.orig_col.push_back((int)(en.first % d.n));
+        const int row = (int)(en.first / d.n), col = (int)(en.first % d.n);
+        p.orig_col.push_back(d.n <= kPackMaxN ? col | row << 16 : col);
         p.orig_code.push_back(en.second);
       }
       for (int a = 0; a < d.n; ++a) loc[p.idx[d.idx_off + a]] = -1;
@@ -316,6 +317,13 @@ std::string build_plan(int nx, int ny, int bx0, int by0, int bw, int bh, int lea
     p.factor_entries += (long long)d.k * d.k + 2LL * d.k * d.m;
   }
   return validate_plan(p);
+}
+
+void flag_interior(Plan* p, int px, int py) {
+  for (int& code : p->orig_code) {
+    const int cell = code / 5, i = cell / p->ny, j = cell - i * p->ny;
+    if (i > px && i < p->nx - 1 - px && j > py && j < p->ny - 1 - py) code |= kInterior;
+  }
 }
 
 std::string validate_plan(const Plan& p) {

@@ -76,8 +76,8 @@ struct Plan {
   std::vector<int> idx;               // grid cells of each front
   std::vector<int> inv;               // extend-add inverse maps
   std::vector<int> orig_ptr;          // per front: n+1 offsets (absolute) into orig_entries
-  std::vector<int> orig_col;          // local column of each original entry
-  std::vector<int> orig_code;         // cell * 5 + direction of each original entry
+  std::vector<int> orig_col;          // local column of each original entry (n <= kPackMaxN: | local row << 16)
+  std::vector<int> orig_code;         // cell * 5 + direction of each original entry (| kInterior, flag_interior)
   std::vector<int> pos;               // elimination position of each grid cell
   int n_levels = 0;
   std::vector<std::vector<int>> level_fronts;  // front ids per level
@@ -95,6 +95,11 @@ struct Plan {
 
 // Builds the plan.  Returns an empty string on success, otherwise an error message.
 std::string build_plan(int nx, int ny, int bx0, int by0, int bw, int bh, int leaf_area, Plan* out);
+
+// Marks the original entries of rows between the absorbing layers (px, py cells on each side), whose
+// couplings are all -1, with kInterior: their values take no table.
+constexpr int kInterior = (int)0x80000000u;
+void flag_interior(Plan* p, int px, int py);
 
 // Checks the plan's invariants (every original entry assembled once, injective
 // extend-add maps, boundary eliminated after pivots).  Empty string when valid.
