@@ -777,6 +777,7 @@ fdfd_status ensure_runtime(fdfd_ctx* ctx) {
   if (ctx->device < 0) {
     CK(cudaGetDevice(&ctx->device));
     CK(factor_init_attributes());
+    CK(panel_init_attributes());
     CK(tc_init_attributes());
     CK(solve_init_attributes());
     CK(dalloc(&ctx->d_cxm, sizeof(double2) * ctx->n_omega * ctx->nx));
@@ -956,9 +957,10 @@ fdfd_status factor_levels(fdfd_ctx* ctx, bool design_only, int w0 = 0, int nw = 
         }
       if (local_piv) {
         {
-          // block LU and inverses, L columns, U rows and the row permutation of the step in one launch
-          Prof pr(ctx, PK_LU_STEP, (pf + lf + tf) * nwd, (pb + lb + tb) * nwd);
-          launch_lu_step_local<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
+          // block LU and inverses, L columns and U rows of the step (LU form: with the panel's update)
+          Prof pr(ctx, PK_LU_STEP, (pf + lf + tf + (sym ? 0 : gf)) * nwd, (pb + lb + tb + (sym ? 0 : gb)) * nwd);
+          if (sym) launch_lu_step_local<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
+          else launch_panel_step<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
         }
         // block row J of L11^-1 and block column J of U11^-1: products with the
         // inverse so far, then with the block's own inverse
@@ -988,7 +990,10 @@ fdfd_status factor_levels(fdfd_ctx* ctx, bool design_only, int w0 = 0, int nw = 
         { Prof pr(ctx, PK_LU_TRSM, tf * nwd, tb * nwd);
           launch_lu_trsm<T>(fa, fl, ll.nlarge, j0, nb, ll.nmax_large, s); }
       }
-      { Prof pr(ctx, PK_LU_GEMM, gf * nwd, gb * nwd); launch_lu_gemm<T>(fa, fl, ll.nlarge, j0, nb, ll.nmax_large, s); }
+      if (!local_piv || sym) {
+        Prof pr(ctx, PK_LU_GEMM, gf * nwd, gb * nwd);
+        launch_lu_gemm<T>(fa, fl, ll.nlarge, j0, nb, ll.nmax_large, s);
+      }
     }
     if (trsm_tc && ll.ntqf > 0) {
       // L21 = F21 U11^-1 and U12 = L11^-1 (P F12) on the tensor cores: the inverse folds of

@@ -49,6 +49,36 @@ template <typename T> __device__ __forceinline__ typename RealOf<T>::type cabs2(
 template <typename T> __device__ __forceinline__ T cscale(T a, typename RealOf<T>::type s) {
   a.x *= s; a.y *= s; return a;
 }
+// max that lets a NaN win, so that a poisoned front is always flagged
+template <typename R>
+__device__ __forceinline__ R nanmax(R a, R b) {
+  if (a != a) return a;
+  if (b != b) return b;
+  return a > b ? a : b;
+}
+
+// complex value of lane src, for every lane of the warp
+template <typename T>
+__device__ __forceinline__ T shfl_c(T v, int src) {
+  v.x = __shfl_sync(0xffffffffu, v.x, src);
+  v.y = __shfl_sync(0xffffffffu, v.y, src);
+  return v;
+}
+
+// 1 / z for a pivot: conj(z) / |z|^2 with the hardware reciprocal estimate of
+// |z|^2 refined by one Newton-Raphson step (double: the correctly rounded one); pivots are far from the over- and underflow range, a zero pivot gives inf / NaN,
+// flagged as growth
+__device__ __forceinline__ float2 pivot_rcp(float2 z) {
+  const float dd = z.x * z.x + z.y * z.y;
+  float s0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s0) : "f"(dd));
+  const float sc = fmaf(s0, fmaf(-dd, s0, 1.0f), s0);
+  return make_float2(z.x * sc, -z.y * sc);
+}
+__device__ __forceinline__ double2 pivot_rcp(double2 z) {
+  const double s = __drcp_rn(z.x * z.x + z.y * z.y);
+  return make_double2(z.x * s, -z.y * s);
+}
 // 1 / (a + ib) by Smith's algorithm (R. L. Smith, CACM 5(8), 1962): scale by the
 // larger component first so that neither the square nor the quotient overflows.
 template <typename T> __device__ __forceinline__ T crcp(T z) {

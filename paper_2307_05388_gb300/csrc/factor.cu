@@ -128,22 +128,6 @@ build_kernel(FactorLaunch a, const int2* __restrict__ tasks) {
   }
 }
 
-// max that lets a NaN win, so that a poisoned front is always flagged
-template <typename R>
-__device__ __forceinline__ R nanmax(R a, R b) {
-  if (a != a) return a;
-  if (b != b) return b;
-  return a > b ? a : b;
-}
-
-// complex value of lane src, for every lane of the warp
-template <typename T>
-__device__ __forceinline__ T shfl_c(T v, int src) {
-  v.x = __shfl_sync(0xffffffffu, v.x, src);
-  v.y = __shfl_sync(0xffffffffu, v.y, src);
-  return v;
-}
-
 // warp argmax of |v|^2 with ties going to the smaller index
 template <typename R>
 __device__ __forceinline__ void warp_argmax(R& v, int& i) {
@@ -200,24 +184,6 @@ __device__ __forceinline__ T pick_slot(const T (&v)[KS], int q) {
     if (q == t) r = v[t];
   return r;
 }
-
-// 1 / z as conj(z) / |z|^2 with a correctly rounded reciprocal (pivots here are
-// far from the over/underflow range; a zero pivot gives inf/NaN, flagged as growth)
-__device__ __forceinline__ double2 fast_crcp(double2 z) {
-  const double s = __drcp_rn(z.x * z.x + z.y * z.y);
-  return make_double2(z.x * s, -z.y * s);
-}
-
-// 1 / z for a pivot: conj(z) / |z|^2 with the hardware reciprocal estimate of
-// |z|^2 refined by one Newton-Raphson step (double: the correctly rounded one)
-__device__ __forceinline__ float2 pivot_rcp(float2 z) {
-  const float dd = z.x * z.x + z.y * z.y;
-  float s0;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s0) : "f"(dd));
-  const float sc = fmaf(s0, fmaf(-dd, s0, 1.0f), s0);
-  return make_float2(z.x * sc, -z.y * sc);
-}
-__device__ __forceinline__ double2 pivot_rcp(double2 z) { return fast_crcp(z); }
 
 // argmax key of a pivot candidate in row r < 128: |v|^2 (as float) with its 7
 // low bits replaced by 127 - r; 0 means no candidate
@@ -1047,55 +1013,44 @@ lu_panel_reg_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int n
 }
 
 // ---------------------------------------------------------------------------
-// Block-local pivoting: one launch per panel step does everything that depends
-// only on the 32 x 32 diagonal block B = F[J, J], J = [j0, j0 + nb):
-//   every CTA LU-factors B itself (warps 0-3, rows in registers, pivot rows
-//   chosen inside B; deterministic, so every CTA gets the same bits) while
+// Symmetric form: one launch per panel step does everything that depends only
+// on the 32 x 32 diagonal block B = F[J, J], J = [j0, j0 + nb):
+//   every CTA LU-factors B itself (warps 0-3, rows in registers, the pivots the
+//   diagonal in order; deterministic, so every CTA gets the same bits) while
 //   warps 4-7 stage the CTA's operand, then does one role:
-//     role D (block 0): the row permutation of J into perm, L_JJ^-1 and U_JJ^-1
+//     role D (block 0): the identity into perm, L_JJ^-1 and U_JJ^-1
 //                       into the diagonal block of the inverse store (L_JJ^-1
 //                       strictly below the diagonal, U_JJ^-1 on and above it),
 //                       growth of its multipliers;
-//     role L: rows r >= j0 + nb, L[r, J] U_JJ = F[r, J]          (64 rows / CTA);
-//     role U: columns c >= j0 + nb, L_JJ U[J, c] = (P F)[J, c]   (64 columns / CTA);
-//     role P: columns c < j0, F[J, c] <- (P F)[J, c]             (64 columns / CTA);
-//   L and U by one-thread-per-row/column substitution against the factored B.
+//     role L: rows r >= j0 + nb, L[r, J] U_JJ = F[r, J]          (256 rows / CTA),
+//             by one-thread-per-row substitution against the factored B.
 // The factored diagonal block is not stored back into F (nothing reads it there:
 // the sweeps and lu_inv_fold use the inverse store).  Roles touch disjoint
-// entries of F and read B only, so the CTAs are independent.
+// entries of F and read B only, so the CTAs are independent.  (The LU form's
+// steps: panel.cu.)
 // ---------------------------------------------------------------------------
-constexpr int kStepRows = 256;   // roles L and U: rows / columns per CTA, one per thread
-constexpr int kStepCols = 64;    // role P: columns per CTA
-static_assert(kStepRows == 1 << 8 && kStepCols == 1 << 6, "the staging loops shift by 8 and 6");
+constexpr int kStepRows = 256;   // role L: rows per CTA, one per thread
 
-// LU of the nb x nb block at (j0, j0) with row pivoting inside the block, by
-// warps 0-3 (lane = row; warp w holds columns 8w..8w+7 in registers).  No rows
-// are swapped: at step p the warp owning column p picks the unused lane r with
-// the largest |a_p| (one redux over packed keys: |a_p|^2 in the high bits,
-// 31 - lane in the low 5, so ties go to the lower lane) and publishes r and
-// every lane's multiplier through shared memory (double-buffered, one 128-thread
-// named barrier per step); each warp then updates its own columns.  On return
-// (after the caller's __syncthreads) LU[p] holds row p of L\U in pivot order,
-// src[p] the block row it came from, dinv[p] = 1 / U[p][p].  Returns this
-// lane's largest |multiplier|^2 (NaN -> inf).
+// LU of the nb x nb block at (j0, j0) without pivoting (only its lower triangle is
+// current: read mirrored), by warps 0-3 (lane = row; warp w holds columns
+// 8w..8w+7 in registers): the warp owning column p publishes every lane's
+// multiplier through shared memory (double-buffered, one 128-thread named
+// barrier per step); each warp then updates its own columns.  On return (after
+// the caller's __syncthreads) LU[p] holds row p of L\U, dinv[p] = 1 / U[p][p].
+// Returns this lane's largest |multiplier|^2 (NaN -> inf).
 template <typename T>
 __device__ __forceinline__ typename RealOf<T>::type diag_lu_4warps(const T* __restrict__ F, int ld, int j0, int nb,
-                                                                   T (*LU)[kMaxNb + 1], int* src, T* dinv,
-                                                                   T (*s_l)[32], int* s_r, bool sym = false) {
+                                                                   T (*LU)[kMaxNb + 1], T* dinv, T (*s_l)[32]) {
   using R = typename RealOf<T>::type;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const T one = cmk(R(1), R(0));
   T a[8];
-  // symmetric form: only the block's lower triangle is current (read it mirrored),
-  // and the pivots are the diagonal in order (no pivoting)
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const int j = 8 * warp + c;
-    const int ri = (sym && j > lane) ? j : lane, ci = (sym && j > lane) ? lane : j;
+    const int ri = j > lane ? j : lane, ci = j > lane ? lane : j;
     a[c] = (lane < nb && j < nb) ? F[(size_t)(j0 + ri) * ld + j0 + ci] : (lane == j ? one : czero<T>());
   }
-  bool used = false;
-  int myp = lane;                 // padding lanes (>= nb) keep their own position
   R g = 0;
   for (int p = 0; p < nb; ++p) {
     const int buf = p & 1, cp = p & 7;
@@ -1104,18 +1059,11 @@ __device__ __forceinline__ typename RealOf<T>::type diag_lu_4warps(const T* __re
 #pragma unroll
       for (int c = 1; c < 8; ++c)
         if (c == cp) ap = a[c];
-      const float v = (float)cabs2(ap);
-      const T myinv = pivot_rcp(ap);    // every lane's candidate, formed beside the redux
-      unsigned key = used ? 0u : ((__float_as_uint(v) & ~31u) | (unsigned)(31 - lane));
-      if (!used && !(v == v)) key = 0xffffffe0u | (unsigned)(31 - lane);   // NaN wins
-      if (sym) key = lane == p ? (0xffffffe0u | (unsigned)(31 - lane)) : 0u;   // the diagonal, in order
-      const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
-      const int r = 31 - (int)(kmax & 31u);
-      const T inv = shfl_c(myinv, r);
-      const bool elim = !used && lane != r;
+      const T inv = shfl_c(pivot_rcp(ap), p);
+      const bool elim = lane > p;
       const T l = elim ? cmul(ap, inv) : czero<T>();
       s_l[buf][lane] = l;
-      if (lane == 0) { s_r[buf] = r; src[p] = r; dinv[p] = inv; }
+      if (lane == 0) dinv[p] = inv;
       if (elim) {
 #pragma unroll
         for (int c = 0; c < 8; ++c)
@@ -1123,9 +1071,7 @@ __device__ __forceinline__ typename RealOf<T>::type diag_lu_4warps(const T* __re
       }
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");
-    const int r = s_r[buf];
     const T l = s_l[buf][lane];
-    if (lane == r) { used = true; myp = p; }
     {
       const R a2 = cabs2(l);
       g = (a2 == a2) ? (a2 > g ? a2 : g) : R(INFINITY);
@@ -1133,72 +1079,54 @@ __device__ __forceinline__ typename RealOf<T>::type diag_lu_4warps(const T* __re
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       const int j = 8 * warp + c;
-      const T u = shfl_c(a[c], r);
+      const T u = shfl_c(a[c], p);
       if (j > p) a[c] = cfms(l, u, a[c]);   // l = 0 on the pivot and on used lanes
     }
   }
 #pragma unroll
-  for (int c = 0; c < 8; ++c) LU[myp][8 * warp + c] = a[c];
-  if (lane >= nb && warp == 0) { src[lane] = lane; dinv[lane] = one; }   // padding rows stay in place
+  for (int c = 0; c < 8; ++c) LU[lane][8 * warp + c] = a[c];
+  if (lane >= nb && warp == 0) dinv[lane] = one;
   return g;
 }
 
 // phase 0: every CTA factors the diagonal block itself (one wave or less);
 // phase 1: only the role-0 CTA of each front, which also posts the block's
-//          factors (rows of L\U in pivot order, 1 / U_pp, source rows) to the
-//          front's scratch slot;
+//          factors (rows of L\U, 1 / U_pp) to the front's scratch slot;
 // phase 2: the other roles, which load those factors instead (many waves).
 template <typename T>
 __global__ void __launch_bounds__(256)
-lu_step_local_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nl, int nu, int phase) {
+lu_step_local_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nl, int phase) {
   using R = typename RealOf<T>::type;
   using Blk = T[kMaxNb + 1];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Blk* LU = reinterpret_cast<Blk*>(smem_raw);                  // [32][33]
   T* dinv = reinterpret_cast<T*>(LU + kMaxNb);                 // [32]
   T (*s_l)[32] = reinterpret_cast<T (*)[32]>(dinv + kMaxNb);   // [2][32] multipliers of a step
-  Blk* Ws = reinterpret_cast<Blk*>(s_l + 2);   // [kStepRows][33]: role L rows x J; roles U, P: [c][p];
+  Blk* Ws = reinterpret_cast<Blk*>(s_l + 2);   // [kStepRows][33]: role L rows x J;
                                                // role D its first 64 rows (a phase-1 launch has only those)
-  __shared__ int src[kMaxNb];
-  __shared__ int s_r[2];
   __shared__ R s_g[8];
   const int w = blockIdx.z + a.w0;
   const int f = flist[blockIdx.y];
   const FrontDesc d = a.P.fronts[f];
   if (j0 >= d.k) return;
-  // L rows and U columns up to n; a front whose off-diagonal blocks come from the
+  // L rows up to n; a front whose off-diagonal blocks come from the
   // tensor cores stops at its pivot block
   const int nb = min(kMaxNb, d.k - j0), n = (a.pivonly && a.pivonly[f]) ? d.k : d.n, ld = d.ld;
   const int bx = blockIdx.x + (phase == 2 ? 1 : 0);
   const size_t slot = (size_t)blockIdx.z * a.swp_stride + blockIdx.y;
   T* blk = reinterpret_cast<T*>(a.dblk) + slot * kDiagBlkElems;
-  int* bsrc = a.swp + slot * kSwpInts;
   // role and range; CTAs whose range is empty for this front leave before any work
-  int role, lo = 0;
-  if (bx == 0) {
-    role = 0;
-  } else if (bx <= nl) {
-    role = 1; lo = j0 + nb + (bx - 1) * kStepRows;
-    if (lo >= n) return;
-  } else if (bx <= nl + nu) {
-    role = 2; lo = j0 + nb + (bx - 1 - nl) * kStepRows;
-    if (lo >= n) return;
-  } else {
-    role = 3; lo = (bx - 1 - nl - nu) * kStepCols;
-    if (lo >= j0) return;
-  }
+  const int role = bx == 0 ? 0 : 1, lo = j0 + nb + (bx - 1) * kStepRows;
+  if (role == 1 && lo >= n) return;
   T* F = reinterpret_cast<T*>(a.store) + (size_t)w * a.store_stride + d.st_off;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   R g = 0;
   if (warp < 4) {
     if (phase == 2) {
       for (int e = tid; e < kMaxNb * kMaxNb; e += 128) LU[e >> 5][e & 31] = blk[e];
-      if (tid < kMaxNb) {
-        dinv[tid] = blk[kMaxNb * kMaxNb + tid];
-        src[tid] = bsrc[tid];
-      }
+      if (tid < kMaxNb) dinv[tid] = blk[kMaxNb * kMaxNb + tid];
     } else {
-      g = diag_lu_4warps<T>(F, ld, j0, nb, LU, src, dinv, s_l, s_r, a.sym != 0);
+      g = diag_lu_4warps<T>(F, ld, j0, nb, LU, dinv, s_l);
     }
   } else if (role == 1) {
     // meanwhile warps 4-7 stage rows [lo, lo + kStepRows) of the block columns
@@ -1206,30 +1134,19 @@ lu_step_local_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int 
       const int rr = e >> 5, l = e & 31, r = lo + rr;
       Ws[rr][l] = (r < n && l < nb) ? F[(size_t)r * ld + j0 + l] : czero<T>();
     }
-  } else if (role >= 2) {
-    // ... or the block rows (not yet permuted) over columns [lo, lo + width)
-    const int hi = role == 2 ? n : j0;
-    const int lw = role == 2 ? 8 : 6;   // log2 of the width: kStepRows (role U) or kStepCols (role P)
-    for (int e = tid - 128; e < (kMaxNb << lw); e += 128) {
-      const int p = e >> lw, cc = e & ((1 << lw) - 1), c = lo + cc;
-      Ws[cc][p] = (c < hi && p < nb) ? F[(size_t)(j0 + p) * ld + c] : czero<T>();
-    }
   }
   __syncthreads();
   if (phase == 1) {
     for (int e = tid; e < kMaxNb * kMaxNb; e += blockDim.x) blk[e] = LU[e >> 5][e & 31];
-    if (tid < kMaxNb) {
-      blk[kMaxNb * kMaxNb + tid] = dinv[tid];
-      bsrc[tid] = src[tid];
-    }
+    if (tid < kMaxNb) blk[kMaxNb * kMaxNb + tid] = dinv[tid];
   }
   // Role D: warp 0 (lane = column c) solves L_JJ x = e_c, warp 1
-  // (lane = row r) solves x U_JJ = e_r, with the same substitution code as roles
-  // U and L; the columns of L_JJ^-1 and rows of U_JJ^-1 meet in the staging tile.
+  // (lane = row r) solves x U_JJ = e_r, with the same substitution code as role
+  // L; the columns of L_JJ^-1 and rows of U_JJ^-1 meet in the staging tile.
   const T one = cmk(R(1), R(0));
   const bool sub_up = (role == 1 && tid < kStepRows) || (role == 0 && warp == 1);
-  const bool sub_lo = (role == 2 && tid < kStepRows) || (role == 0 && warp == 0);
-  if (role == 0 && tid < nb) a.perm[(size_t)w * a.perm_stride + d.piv_off + j0 + tid] = j0 + src[tid];
+  const bool sub_lo = role == 0 && warp == 0;
+  if (role == 0 && tid < nb) a.perm[(size_t)w * a.perm_stride + d.piv_off + j0 + tid] = j0 + tid;
   if (sub_up) {
     // x U_JJ = b: one thread per row, right-looking substitution
     T x[kMaxNb];
@@ -1261,31 +1178,13 @@ lu_step_local_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int 
     // L_JJ x = b: one thread per column, unit-lower substitution
     T x[kMaxNb];
 #pragma unroll
-    for (int i = 0; i < kMaxNb; ++i) x[i] = role == 2 ? Ws[tid][src[i]] : (i == lane ? one : czero<T>());
+    for (int i = 0; i < kMaxNb; ++i) x[i] = i == lane ? one : czero<T>();
 #pragma unroll
     for (int i = 0; i < kMaxNb; ++i)
 #pragma unroll
       for (int ii = i + 1; ii < kMaxNb; ++ii) x[ii] = cfms(LU[ii][i], x[i], x[ii]);
-    if (role == 2) {
-      // U[J, c] = L_JJ^-1 (P F)[J, c]
-      const int c = lo + tid;
-      if (c < n)
 #pragma unroll
-        for (int i = 0; i < kMaxNb; ++i)
-          if (i < nb) F[(size_t)(j0 + i) * ld + c] = x[i];
-    } else {
-#pragma unroll
-      for (int i = 0; i < kMaxNb; ++i) Ws[i][lane] = x[i];             // column lane of L_JJ^-1
-    }
-  } else if (role == 3) {
-    // role P: (P F)[i][c] for the columns left of the block
-    const int cc = tid & 63, ig = tid >> 6;
-    const int c = lo + cc;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int i = ig + 4 * q;
-      if (c < j0 && i < nb) F[(size_t)(j0 + i) * ld + c] = Ws[cc][src[i]];
-    }
+    for (int i = 0; i < kMaxNb; ++i) Ws[i][lane] = x[i];               // column lane of L_JJ^-1
   }
   if (role == 0) {
     // the diagonal block of the inverse store: L_JJ^-1 strictly below the
@@ -1297,7 +1196,7 @@ lu_step_local_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int 
       X[(size_t)(j0 + i) * d.ldk + j0 + j] = i > j ? Ws[i][j] : Ws[kMaxNb + i][j];
     }
   }
-  if (role <= 1) {
+  {
     for (int o = 16; o > 0; o >>= 1) g = nanmax(g, __shfl_xor_sync(0xffffffffu, g, o));
     if (lane == 0) s_g[warp] = g;
     __syncthreads();
@@ -1607,6 +1506,14 @@ lu_inv_fold_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nq
   T* X = reinterpret_cast<T*>(a.istore) + (size_t)w * a.istore_stride + d.iv_off;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const T one = cmk(R(1), R(0));
+  // rows of L[J, :]: where the factorisation left them (the panel steps do not move earlier columns)
+  const int* Pm = a.perm + (size_t)w * a.perm_stride + d.piv_off;
+  int lrow[4];
+#pragma unroll
+  for (int qq = 0; qq < 4; ++qq) {
+    const int i = ty + 8 * qq;
+    lrow[qq] = (upper || i >= nb) ? j0 : a.sym ? j0 + i : Pm[j0 + i];
+  }
   // element e = ty + 8 q' of this thread's four: row (ty + 8 q'), column tx of a slice
   auto fetch = [&](int l0, T* ra, T* rb) {
 #pragma unroll
@@ -1615,7 +1522,7 @@ lu_inv_fold_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nq
       const int la = l0 + tx;            // A[i][tx]: column l of the left operand
       T va = czero<T>();
       if (la < j0) {
-        if (!upper) va = i < nb ? F[(size_t)(j0 + i) * ld + la] : czero<T>();
+        if (!upper) va = i < nb ? F[(size_t)lrow[qq] * ld + la] : czero<T>();
         else {
           const int r = c0 + i;
           va = (la >= r) ? X[(size_t)r * ldk + la] : czero<T>();
@@ -1886,9 +1793,7 @@ void launch_lu_step_local(const FactorLaunch& a, const int* flist, int nf, int j
   if (nf <= 0) return;
   const int span = std::max(0, nmax - j0 - 1);
   const int nl = (span + kStepRows - 1) / kStepRows;
-  // symmetric form: no U rows (the trailing update takes diag(d) L^T instead) and no row permutation
-  const int nu = a.sym ? 0 : nl;
-  const int np = a.sym ? 0 : (j0 + kStepCols - 1) / kStepCols;
+  // (no U rows: the trailing update takes diag(d) L^T instead)
   // CTAs resident at once on the current device
   int dev = 0, nsm = 0, per_sm = 0;
   const long long wave =
@@ -1897,17 +1802,17 @@ void launch_lu_step_local(const FactorLaunch& a, const int* flist, int nf, int j
            cudaSuccess)
           ? (long long)std::max(1, per_sm) * nsm
           : (1LL << 40);
-  const long long ctas = (long long)(1 + nl + nu + np) * nf * a.n_omega;
+  const long long ctas = (long long)(1 + nl) * nf * a.n_omega;
   if (ctas > wave && a.dblk) {
     // more than one wave: the diagonal block once per front (four warps: the block LU, then
     // role D; a smaller footprint, so that more fronts share an SM), then the substitutions
-    lu_step_local_kernel<T><<<dim3(1, nf, a.n_omega), 128, step_diag_smem(sizeof(T)), s>>>(a, flist, j0, nl, nu, 1);
-    if (nl + nu + np > 0)
-      lu_step_local_kernel<T><<<dim3(nl + nu + np, nf, a.n_omega), 256, step_local_smem(sizeof(T)), s>>>(
-          a, flist, j0, nl, nu, 2);
+    lu_step_local_kernel<T><<<dim3(1, nf, a.n_omega), 128, step_diag_smem(sizeof(T)), s>>>(a, flist, j0, nl, 1);
+    if (nl > 0)
+      lu_step_local_kernel<T><<<dim3(nl, nf, a.n_omega), 256, step_local_smem(sizeof(T)), s>>>(
+          a, flist, j0, nl, 2);
   } else {
-    lu_step_local_kernel<T><<<dim3(1 + nl + nu + np, nf, a.n_omega), 256, step_local_smem(sizeof(T)), s>>>(
-        a, flist, j0, nl, nu, 0);
+    lu_step_local_kernel<T><<<dim3(1 + nl, nf, a.n_omega), 256, step_local_smem(sizeof(T)), s>>>(
+        a, flist, j0, nl, 0);
   }
 }
 

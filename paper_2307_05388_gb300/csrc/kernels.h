@@ -57,12 +57,15 @@ template <typename T> void launch_lu_panel(const FactorLaunch& a, const int* fli
                                            int nb, int kmax, cudaStream_t s);
 template <typename T> void launch_lu_l21(const FactorLaunch& a, const int* flist, int nf, int j0,
                                          int nb, int mmax, int nmax, int below, cudaStream_t s);
-// Pivoting restricted to the 32 x 32 diagonal block J = [j0, j0 + 32): one launch
-// does the block's LU, the L columns below it, the U rows right of it, the row
-// permutation of earlier columns and perm, and writes L_JJ^-1 / U_JJ^-1 into the
-// diagonal block of the inverse store; then launch_lu_gemm does the trailing
-// update and launch_lu_inv_fold the rest of block row / column J of the inverses.
-// nmax = largest n listed.
+// Panel step with pivoting restricted to the 32 x 32 diagonal block J = [j0, j0 + 32): the block's LU, the
+// L columns below it, the U rows right of it and perm, L_JJ^-1 / U_JJ^-1 into the diagonal block of the
+// inverse store; launch_lu_inv_fold does the rest of block row / column J of the inverses.
+// nmax = largest n listed, the same for every step of a level.
+// LU form (panel.cu): left-looking, no trailing update follows; earlier columns' rows are not permuted.
+template <typename T> void launch_panel_step(const FactorLaunch& a, const int* flist, int nf, int j0, int nmax,
+                                             cudaStream_t s);
+cudaError_t panel_init_attributes();
+// Symmetric form (no pivoting; L columns only): launch_lu_gemm does the trailing update.
 template <typename T> void launch_lu_step_local(const FactorLaunch& a, const int* flist, int nf, int j0,
                                                 int nmax, cudaStream_t s);
 constexpr int kSwapScratchInts = 130;   // ints of swap scratch per (wavelength, listed front)
@@ -122,7 +125,7 @@ cudaError_t launch_mbar_probe(int* err, cudaStream_t s);
 template <typename T> void launch_lu_gemm(const FactorLaunch& a, const int* flist, int nf, int j0,
                                           int nb, int nmax, cudaStream_t s);
 // block row J of L11^-1 and block column J of U11^-1 (J = [j0, j0 + 32)) after
-// launch_lu_step_local wrote the diagonal block J and the folds of
+// the panel step wrote the diagonal block J and the folds of
 // the earlier blocks are done; reads only entries that no later step writes, so
 // it may run beside the front's later steps.
 template <typename T> void launch_lu_inv_fold(const FactorLaunch& a, const int* flist, int nf, int j0,
