@@ -243,6 +243,88 @@ __device__ __forceinline__ void write_pack_rows(T* __restrict__ B, int m, int k,
     for (int c = c0; c < ks; c += 1 << lw) B[t * ks + c] = c < k ? val(t, c) : czero<T>();
 }
 
+// The packed triangular inverses of a small front, four rows of each at a time per warp: lane holds
+// columns lane + 32 q (k <= 32 KS).  Starting from rows of the identity, pivot m's step is nothing for the rows
+// it does not reach; one load of the factor's row serves four rows, whose chains overlap.
+template <typename T, int NWARP, int KS>
+__device__ __forceinline__ void small_inverses(const T* S, int ls, int k, const int* s_pm, T* __restrict__ Lb,
+                                               T* __restrict__ Ub, int warp, int lane) {
+  using R = typename RealOf<T>::type;
+  constexpr int kRows = 4;
+  T dinv[KS];
+#pragma unroll
+  for (int q = 0; q < KS; ++q) {
+    const int c = lane + 32 * q;
+    dinv[q] = c < k ? pivot_rcp(S[s_pm[c] * ls + c]) : czero<T>();
+  }
+#pragma unroll 1
+  for (int i0 = kRows * warp; i0 < k; i0 += kRows * NWARP) {
+    T acc[kRows][KS];
+    auto identity = [&]() {
+#pragma unroll
+      for (int r = 0; r < kRows; ++r)
+#pragma unroll
+        for (int q = 0; q < KS; ++q) acc[r][q] = cmk(lane + 32 * q == i0 + r ? R(1) : R(0), R(0));
+    };
+    // rows of L11^-1, columns l < i
+    identity();
+#pragma unroll
+    for (int qs = KS - 1; qs >= 0; --qs) {
+      const int hi = min(min(i0 + kRows - 1, k - 1), 32 * qs + 31);
+#pragma unroll 2
+      for (int m = hi; m >= max(1, 32 * qs); --m) {
+        const T* Lm = S + s_pm[m] * ls;
+        T y[kRows], v[KS];
+#pragma unroll
+        for (int q = 0; q <= qs; ++q) v[q] = lane + 32 * q < m ? Lm[lane + 32 * q] : czero<T>();
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) y[r] = shfl_c(acc[r][qs], m & 31);
+#pragma unroll
+        for (int q = 0; q <= qs; ++q)
+#pragma unroll
+          for (int r = 0; r < kRows; ++r) acc[r][q] = cfms(y[r], v[q], acc[r][q]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+#pragma unroll
+      for (int q = 0; q < KS; ++q) {
+        const int i = i0 + r, l = lane + 32 * q;
+        if (i < k && l < i) Lb[pack_diag(i - l, k) + l] = acc[r][q];
+      }
+    // rows of U11^-1, columns c >= i
+    identity();
+#pragma unroll
+    for (int qs = 0; qs < KS; ++qs) {
+      const int hi = min(k - 1, 32 * qs + 31);
+#pragma unroll 2
+      for (int l = max(i0, 32 * qs); l <= hi; ++l) {
+        const T* Ul = S + s_pm[l] * ls;
+        const T dl = shfl_c(dinv[qs], l & 31);
+        T y[kRows], v[KS];
+#pragma unroll
+        for (int q = qs; q < KS; ++q) {
+          const int c = lane + 32 * q;
+          v[q] = (c > l && c < k) ? Ul[c] : czero<T>();
+        }
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) y[r] = cmul(shfl_c(acc[r][qs], l & 31), dl);
+#pragma unroll
+        for (int q = qs; q < KS; ++q)
+#pragma unroll
+          for (int r = 0; r < kRows; ++r) acc[r][q] = cfms(y[r], v[q], acc[r][q]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+#pragma unroll
+      for (int q = 0; q < KS; ++q) {
+        const int i = i0 + r, c = lane + 32 * q;
+        if (i < k && c >= i && c < k) Ub[pack_diag(c - i, k) + i] = cmul(acc[r][q], dinv[q]);
+      }
+  }
+}
+
 template <typename T, int NWARP, int RI, int RJ, int MINB>
 __global__ void __launch_bounds__(NWARP * 32, MINB)
 lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
@@ -293,17 +375,43 @@ lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
       s_pos[c] = k;
     }
     __syncthreads();
-    // the children's update-matrix rows through their inverse extend-add maps
-#pragma unroll 2
-    for (int r = warp; r < n; r += NWARP) {
-      const int ia = s_i0[r], ib = s_i1[r];
-      const T* S0 = ia >= 0 ? st + c0.st_off + (size_t)(c0.k + ia) * c0.ld + c0.k : nullptr;
-      const T* S1 = ib >= 0 ? st + c1.st_off + (size_t)(c1.k + ib) * c1.ld + c1.k : nullptr;
-      for (int c = lane; c < n; c += 32) {
-        T v = czero<T>();
-        if (S0) { const int i0 = s_i0[c]; if (i0 >= 0) v = cadd(v, S0[i0]); }
-        if (S1) { const int i1 = s_i1[c]; if (i1 >= 0) v = cadd(v, S1[i1]); }
-        S[r * ls + c] = v;
+    // the children's update-matrix rows through their inverse extend-add maps: a lane's columns are the
+    // same in every row, and the loads of kRows rows are in flight together
+    if (nc == 0) {
+      for (int e = tid; e < n * ls; e += THREADS) S[e] = czero<T>();
+    } else {
+      constexpr int kRows = 4, KC = (NMAX + 31) / 32;
+      const T* S0 = st + c0.st_off + (size_t)c0.k * c0.ld + c0.k;
+      const T* S1 = nc > 1 ? st + c1.st_off + (size_t)c1.k * c1.ld + c1.k : S0;
+      const int ld0 = c0.ld, ld1 = nc > 1 ? c1.ld : 0;
+      int i0[KC], i1[KC];
+#pragma unroll
+      for (int q = 0; q < KC; ++q) {
+        const int c = lane + 32 * q;
+        i0[q] = c < n ? s_i0[c] : -1;
+        i1[q] = c < n ? s_i1[c] : -1;
+      }
+#pragma unroll 1
+      for (int r0 = warp; r0 < n; r0 += kRows * NWARP) {
+        T v0[kRows][KC], v1[kRows][KC];
+#pragma unroll
+        for (int b = 0; b < kRows; ++b) {
+          const int r = r0 + b * NWARP;
+          const int ia = r < n ? s_i0[r] : -1, ib = r < n ? s_i1[r] : -1;
+#pragma unroll
+          for (int q = 0; q < KC; ++q) {
+            v0[b][q] = v1[b][q] = czero<T>();
+            if ((ia | i0[q]) >= 0) v0[b][q] = S0[ia * ld0 + i0[q]];
+            if ((ib | i1[q]) >= 0) v1[b][q] = S1[ib * ld1 + i1[q]];
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < kRows; ++b) {
+          const int r = r0 + b * NWARP;
+#pragma unroll
+          for (int q = 0; q < KC; ++q)
+            if (r < n && lane + 32 * q < n) S[r * ls + lane + 32 * q] = cadd(v0[b][q], v1[b][q]);
+        }
       }
     }
     __syncthreads();
@@ -368,15 +476,19 @@ lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
           gmax = nanmax(gmax, cabs2(l[i]));
         }
     }
-    // every column of the unused rows: the ones up to j are below the row's own
-    // pivot step (or < k), so they are never written back
+    // the unused rows, four of the warp's columns at a time while one of them is right of j (columns up to
+    // j are below the row's own pivot step, or < k, and never written back)
 #pragma unroll
-    for (int jj = 0; jj < RJ; ++jj) {
-      const T u = s_u[warp][jj];
+    for (int j4 = 0; j4 < RJ; j4 += 4)
+      if (j < warp + NWARP * (j4 + 3)) {
 #pragma unroll
-      for (int i = 0; i < RI; ++i)
-        if (act[i]) x[i][jj] = cfms(l[i], u, x[i][jj]);
-    }
+        for (int jj = j4; jj < j4 + 4; ++jj) {
+          const T u = s_u[warp][jj];
+#pragma unroll
+          for (int i = 0; i < RI; ++i)
+            if (act[i]) x[i][jj] = cfms(l[i], u, x[i][jj]);
+        }
+      }
     if (j + 1 < k && warp == (j + 1) % NWARP)
       small_post_column<T, RI, RJ>(x, done, (j + 1) / NWARP, n, k, lane, s_col[par ^ 1], &s_key[par ^ 1]);
     __syncthreads();
@@ -394,55 +506,11 @@ lu_small_kernel(FactorLaunch a, const int* __restrict__ flist) {
     }
   }
   __syncthreads();
-  // triangular inverses, rows i = warp, warp + NWARP, ...; lane holds columns lane + 32 q (KS slots: k <= 32 KS)
-  constexpr int KS = (NMAX + 31) / 32;
   T* Lb = reinterpret_cast<T*>(a.pack) + (size_t)w * a.pack_stride + d.pk_off;   // the front's packed blocks
   T* Ub = Lb + a.pack_stride / 2;
-  const T one = cmk(R(1), R(0));
-  T dinv[KS];
-#pragma unroll
-  for (int q = 0; q < KS; ++q) {
-    const int c = lane + 32 * q;
-    dinv[q] = c < k ? pivot_rcp(S[s_pm[c] * ls + c]) : czero<T>();
-  }
-  for (int i = warp; i < k; i += NWARP) {
-    T acc[KS];
-    // row i of L11^-1, columns l < i
-#pragma unroll
-    for (int q = 0; q < KS; ++q) acc[q] = czero<T>();
-    for (int m = i; m >= 1; --m) {
-      const T ym = m == i ? one : shfl_c(pick_slot<T, KS>(acc, m >> 5), m & 31);
-      const T* Lm = S + s_pm[m] * ls;
-#pragma unroll
-      for (int q = 0; q < KS; ++q) {
-        const int l = lane + 32 * q;
-        if (l < m) acc[q] = cfms(ym, Lm[l], acc[q]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < KS; ++q) {
-      const int l = lane + 32 * q;
-      if (l < i) Lb[pack_diag(i - l, k) + l] = acc[q];
-    }
-    // row i of U11^-1, columns c >= i
-#pragma unroll
-    for (int q = 0; q < KS; ++q) acc[q] = (lane + 32 * q == i) ? one : czero<T>();
-    for (int l = i; l < k; ++l) {
-      const int q = l >> 5;
-      const T yl = shfl_c(cmul(pick_slot<T, KS>(acc, q), pick_slot<T, KS>(dinv, q)), l & 31);
-      const T* Ul = S + s_pm[l] * ls;
-#pragma unroll
-      for (int qq = 0; qq < KS; ++qq) {
-        const int c = lane + 32 * qq;
-        if (c > l && c < k) acc[qq] = cfms(yl, Ul[c], acc[qq]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < KS; ++q) {
-      const int c = lane + 32 * q;
-      if (c >= i && c < k) Ub[pack_diag(c - i, k) + i] = cmul(acc[q], dinv[q]);
-    }
-  }
+  if (NMAX <= 32 || k <= 32) small_inverses<T, NWARP, 1>(S, ls, k, s_pm, Lb, Ub, warp, lane);
+  else if (NMAX <= 64 || k <= 64) small_inverses<T, NWARP, 2>(S, ls, k, s_pm, Lb, Ub, warp, lane);
+  else small_inverses<T, NWARP, 3>(S, ls, k, s_pm, Lb, Ub, warp, lane);
   // the update matrix, the packed off-diagonal blocks, the permutation, the growth
   for (int r = k + warp; r < n; r += NWARP) {
     const T* Sr = S + r * ls;
