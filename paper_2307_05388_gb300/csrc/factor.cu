@@ -1543,30 +1543,29 @@ template <typename T> struct GemmKc;
 template <> struct GemmKc<float2> { static constexpr int v = 32; };
 template <> struct GemmKc<double2> { static constexpr int v = 16; };
 
-// Two uses (SIMT complex FMA, 64 x 64 tiles):
-//   schur = 0: panel step at j0 -- trailing update restricted to the pivot-block
-//              rows and columns; the m x m update matrix S is left untouched
-//   schur = 1: once per front after its last panel -- S = F22 - L21 U12, K = k
 // Block row J of L11^-1 and block column J of U11^-1 of the listed large fronts,
 // once the diagonal block J of the inverse store holds L_JJ^-1 / U_JJ^-1 and
 // every block before J is done (block-local pivoting: rows of J never move
 // again, and nothing later writes the entries read here):
-//   lower, columns c in [c0, c0 + 32):  X[J][c] = -L_JJ^-1  sum_{l in [c, j0)} L[J][l] X[l][c]   (from L X = I)
-//   upper, rows r in [r0, r0 + 32):     X[r][J] = -(sum_{l in [r, j0)} X[r][l] U[l][J]) U_JJ^-1 (from X U = I)
-// One CTA per (32-wide chunk, triangle, front): blockIdx.x < nq lower chunk
+//   lower, columns c in [c0, c0 + CW):  X[J][c] = -L_JJ^-1  sum_{l in [c, j0)} L[J][l] X[l][c]   (from L X = I)
+//   upper, rows r in [r0, r0 + CW):     X[r][J] = -(sum_{l in [r, j0)} X[r][l] U[l][J]) U_JJ^-1 (from X U = I)
+// One CTA per (CW-wide chunk, triangle, front): blockIdx.x < nq lower chunk
 // q = blockIdx.x, else upper chunk q = blockIdx.x - nq.  The contraction runs
 // over 32-wide slices of l with the next slice prefetched into registers.
-template <typename T>
+// CW = 32 reuses each operand of a slice over 32; CW = 8 spreads a fold over four times the CTAs
+// (the rule: launch_lu_inv_fold).
+template <typename T, int CW>
 __global__ void __launch_bounds__(256)
 lu_inv_fold_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nq) {
-  __shared__ T Am[32][33];   // left operand slice, then T (the sum)
-  __shared__ T Bm[32][33];   // right operand slice, then the diagonal inverse block
+  constexpr int Q = 32 * CW / 256, TR = 256 / CW;    // outputs per thread; lower: rows a pass of the CTA covers
+  __shared__ T Bq[32][33];   // the 32 x 32 operand: L[J][slice] or U[slice][J], then the diagonal inverse block
+  __shared__ T Cq[32 * (CW + 1)];   // the chunk's: X[slice][chunk] (rows of CW + 1) or X[chunk][slice] (of 33), then the sums
   using R = typename RealOf<T>::type;
   const int w = blockIdx.z + a.w0;
   const FrontDesc d = a.P.fronts[flist[blockIdx.y]];
   if (j0 >= d.k) return;
   const bool upper = (int)blockIdx.x >= nq;
-  const int c0 = (upper ? (int)blockIdx.x - nq : (int)blockIdx.x) * 32;
+  const int c0 = (upper ? (int)blockIdx.x - nq : (int)blockIdx.x) * CW;
   if (c0 >= j0) return;
   const int nb = min(kMaxNb, d.k - j0);
   const int ld = d.ld, ldk = d.ldk;
@@ -1574,6 +1573,9 @@ lu_inv_fold_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nq
   T* X = reinterpret_cast<T*>(a.istore) + (size_t)w * a.istore_stride + d.iv_off;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const T one = cmk(R(1), R(0));
+  // this thread's outputs: lower (oi + TR q, oj) of J x chunk, upper (oi + 8 q, oj) of chunk x J
+  const int oi = upper ? ty : tid / CW, oj = upper ? tx : tid % CW, os = upper ? 8 : TR;
+  const int cs = upper ? 33 : CW + 1;                // row stride of Cq
   // rows of L[J, :]: where the factorisation left them (the panel steps do not move earlier columns)
   const int* Pm = a.perm + (size_t)w * a.perm_stride + d.piv_off;
   int lrow[4];
@@ -1582,90 +1584,100 @@ lu_inv_fold_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nq
     const int i = ty + 8 * qq;
     lrow[qq] = (upper || i >= nb) ? j0 : a.sym ? j0 + i : Pm[j0 + i];
   }
-  // element e = ty + 8 q' of this thread's four: row (ty + 8 q'), column tx of a slice
-  auto fetch = [&](int l0, T* ra, T* rb) {
+  auto fetch = [&](int l0, T* rb, T* rc) {
 #pragma unroll
     for (int qq = 0; qq < 4; ++qq) {
       const int i = ty + 8 * qq;
-      const int la = l0 + tx;            // A[i][tx]: column l of the left operand
-      T va = czero<T>();
-      if (la < j0) {
-        if (!upper) va = i < nb ? F[(size_t)lrow[qq] * ld + la] : czero<T>();
-        else {
-          const int r = c0 + i;
-          va = (la >= r) ? X[(size_t)r * ldk + la] : czero<T>();
-        }
+      rb[qq] = czero<T>();
+      if (!upper) {
+        if (i < nb && l0 + tx < j0) rb[qq] = F[(size_t)lrow[qq] * ld + l0 + tx];
+      } else {
+        if (l0 + i < j0 && tx < nb) rb[qq] = F[(size_t)(l0 + i) * ld + j0 + tx];
       }
-      ra[qq] = va;
-      const int lb = l0 + i;             // B[i][tx]: row l of the right operand
-      T vb = czero<T>();
-      if (lb < j0) {
-        if (!upper) {
-          const int c = c0 + tx;
-          vb = lb > c ? X[(size_t)lb * ldk + c] : (lb == c ? one : czero<T>());
-        } else {
-          vb = tx < nb ? F[(size_t)lb * ld + j0 + tx] : czero<T>();
-        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int i = oi + os * q;
+      rc[q] = czero<T>();
+      if (!upper) {
+        const int l = l0 + i, c = c0 + oj;
+        if (l < j0) rc[q] = l > c ? X[(size_t)l * ldk + c] : (l == c ? one : czero<T>());
+      } else {
+        const int l = l0 + oj, r = c0 + i;
+        if (l < j0 && l >= r) rc[q] = X[(size_t)r * ldk + l];
       }
-      rb[qq] = vb;
     }
   };
-  T acc[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // T[ty + 8 q'][tx]
-  T ra[4], rb[4];
-  fetch(c0, ra, rb);
+  T acc[Q], rb[4], rc[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) acc[q] = czero<T>();
+  fetch(c0, rb, rc);
   for (int l0 = c0; l0 < j0; l0 += 32) {
 #pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-      Am[ty + 8 * qq][tx] = ra[qq];
-      Bm[ty + 8 * qq][tx] = rb[qq];
-    }
-    __syncthreads();
-    if (l0 + 32 < j0) fetch(l0 + 32, ra, rb);
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      const T bv = Bm[kk][tx];
+    for (int qq = 0; qq < 4; ++qq) Bq[ty + 8 * qq][tx] = rb[qq];
 #pragma unroll
-      for (int qq = 0; qq < 4; ++qq) acc[qq] = cfma(Am[ty + 8 * qq][kk], bv, acc[qq]);
+    for (int q = 0; q < Q; ++q) Cq[(oi + os * q) * cs + oj] = rc[q];
+    __syncthreads();
+    if (l0 + 32 < j0) fetch(l0 + 32, rb, rc);
+    if (!upper) {
+#pragma unroll 8
+      for (int kk = 0; kk < 32; ++kk) {
+        const T v = Cq[kk * cs + oj];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[q] = cfma(Bq[oi + os * q][kk], v, acc[q]);
+      }
+    } else {
+#pragma unroll 8
+      for (int kk = 0; kk < 32; ++kk) {
+        const T v = Bq[kk][oj];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[q] = cfma(Cq[(oi + os * q) * cs + kk], v, acc[q]);
+      }
     }
     __syncthreads();
   }
-  // Am <- T, Bm <- L_JJ^-1 (unit diagonal) or U_JJ^-1, zero outside the block
+  // Cq <- the sums, Bq <- L_JJ^-1 (unit diagonal) or U_JJ^-1, zero outside the block
+#pragma unroll
+  for (int q = 0; q < Q; ++q) Cq[(oi + os * q) * cs + oj] = acc[q];
 #pragma unroll
   for (int qq = 0; qq < 4; ++qq) {
     const int i = ty + 8 * qq, j = tx;
-    Am[i][j] = acc[qq];
     T v = czero<T>();
     if (i < nb && j < nb) {
       if (!upper) v = (j < i) ? X[(size_t)(j0 + i) * ldk + j0 + j] : (i == j ? one : czero<T>());
       else v = (j >= i) ? X[(size_t)(j0 + i) * ldk + j0 + j] : czero<T>();
     }
-    Bm[i][j] = v;
+    Bq[i][j] = v;
   }
   __syncthreads();
 #pragma unroll
-  for (int qq = 0; qq < 4; ++qq) {
-    const int i = ty + 8 * qq;
+  for (int q = 0; q < Q; ++q) {
+    const int i = oi + os * q;
     T o0 = czero<T>(), o1 = czero<T>();
     if (!upper) {
-      // X[J + i][c0 + tx] = -sum_t Li[i][t] T[t][tx]
+      // X[J + i][c0 + oj] = -sum_t Li[i][t] T[t][oj]
 #pragma unroll 8
       for (int t = 0; t < 32; t += 2) {
-        o0 = cfms(Bm[i][t], Am[t][tx], o0);
-        o1 = cfms(Bm[i][t + 1], Am[t + 1][tx], o1);
+        o0 = cfms(Bq[i][t], Cq[t * cs + oj], o0);
+        o1 = cfms(Bq[i][t + 1], Cq[(t + 1) * cs + oj], o1);
       }
-      if (i < nb && c0 + tx < j0) X[(size_t)(j0 + i) * ldk + c0 + tx] = cadd(o0, o1);
+      if (i < nb && c0 + oj < j0) X[(size_t)(j0 + i) * ldk + c0 + oj] = cadd(o0, o1);
     } else {
-      // X[c0 + i][J + tx] = -sum_t T[i][t] Ui[t][tx]
+      // X[c0 + i][J + oj] = -sum_t T[i][t] Ui[t][oj]
 #pragma unroll 8
       for (int t = 0; t < 32; t += 2) {
-        o0 = cfms(Am[i][t], Bm[t][tx], o0);
-        o1 = cfms(Am[i][t + 1], Bm[t + 1][tx], o1);
+        o0 = cfms(Cq[i * cs + t], Bq[t][oj], o0);
+        o1 = cfms(Cq[i * cs + t + 1], Bq[t + 1][oj], o1);
       }
-      if (c0 + i < j0 && tx < nb) X[(size_t)(c0 + i) * ldk + j0 + tx] = cadd(o0, o1);
+      if (c0 + i < j0 && oj < nb) X[(size_t)(c0 + i) * ldk + j0 + oj] = cadd(o0, o1);
     }
   }
 }
 
+// Two uses (SIMT complex FMA, 64 x 64 tiles):
+//   schur = 0: panel step at j0 -- trailing update restricted to the pivot-block
+//              rows and columns; the m x m update matrix S is left untouched
+//   schur = 1: once per front after its last panel -- S = F22 - L21 U12, K = k
 template <typename T>
 __global__ void __launch_bounds__(256)
 lu_gemm_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nbmax, int schur) {
@@ -1914,15 +1926,24 @@ void launch_lu_gemm(const FactorLaunch& a, const int* flist, int nf, int j0, int
 
 template <typename T>
 void launch_lu_inv_fold(const FactorLaunch& a, const int* flist, int nf, int j0, cudaStream_t s) {
-  const int nq = (j0 + 31) / 32;
-  if (nf <= 0 || nq <= 0) return;
+  if (nf <= 0 || j0 <= 0) return;
+  // complex128: its arithmetic bounds a CTA, and 32-wide folds took 70 to 230 us each on a few SMs (the
+  // folds of a 200 x 200 factorisation 1.93 -> 0.60 ms).  complex64 keeps 32: folds of the small levels
+  // would take 0.35 instead of 0.49 ms at 340 x 340, but on more SMs beside the panel steps they run
+  // with, and the pass gets 1% slower.
+  constexpr int CW = sizeof(T) == 8 ? 32 : 8;
+  const int nq = (j0 + CW - 1) / CW;
   // the symmetric form needs L11^-1 only (the first nq CTAs)
-  lu_inv_fold_kernel<T><<<dim3(a.sym ? nq : 2 * nq, nf, a.n_omega), 256, 0, s>>>(a, flist, j0, nq);
+  lu_inv_fold_kernel<T, CW><<<dim3(a.sym ? nq : 2 * nq, nf, a.n_omega), 256, 0, s>>>(a, flist, j0, nq);
 }
 
 template <typename T>
 void launch_schur_simt(const FactorLaunch& a, const int* flist, int nf, int mmax, cudaStream_t s) {
   if (nf <= 0 || mmax <= 0) return;
+  if (sizeof(T) == 16 && !a.sym) {
+    launch_schur_fine(a, flist, nf, mmax, s);
+    return;
+  }
   const int nt = (mmax + kGemmTile - 1) / kGemmTile;
   lu_gemm_kernel<T><<<dim3(nt * nt, nf, a.n_omega), 256, 0, s>>>(a, flist, 0, 0, 1);
 }

@@ -65,6 +65,8 @@ template <typename T> void launch_lu_l21(const FactorLaunch& a, const int* flist
 template <typename T> void launch_panel_step(const FactorLaunch& a, const int* flist, int nf, int j0, int nmax,
                                              cudaStream_t s);
 cudaError_t panel_init_attributes();
+// complex128, LU form: S = F22 - L21 U12 of the listed fronts (mmax = largest m listed)
+void launch_schur_fine(const FactorLaunch& a, const int* flist, int nf, int mmax, cudaStream_t s);
 // Symmetric form (no pivoting; L columns only): launch_lu_gemm does the trailing update.
 template <typename T> void launch_lu_step_local(const FactorLaunch& a, const int* flist, int nf, int j0,
                                                 int nmax, cudaStream_t s);

@@ -670,6 +670,20 @@ panel_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nt, int 
   }
 }
 
+// Update matrix of a complex128 front, S = F22 - L21 U12, in tiles of the panel's products: its arithmetic
+// bounds a CTA, and 64 x 64 tiles left most SMs idle (480 us a launch at 200 x 200, one wavelength;
+// all update matrices of that factorisation 2.57 -> 0.91 ms).
+__global__ void __launch_bounds__(kPanelThreads) schur_fine_kernel(FactorLaunch a, const int* __restrict__ flist, int nt) {
+  constexpr int kT = Shape<double2>::kXt;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int w = blockIdx.z + a.w0;
+  const FrontDesc d = a.P.fronts[flist[blockIdx.y]];
+  const int r0 = d.k + blockIdx.x / nt * kT, c0 = d.k + blockIdx.x % nt * kT;
+  if (r0 >= d.n || c0 >= d.n) return;
+  double2* F = reinterpret_cast<double2*>(a.store) + (size_t)w * a.store_stride + d.st_off;
+  panel_product<double2, kT, kT, 1>(F, d.ld, r0, d.n, c0, d.n, d.k, smem_raw);
+}
+
 template <typename T, int PHASE>
 cudaError_t panel_attribute() {
   return cudaFuncSetAttribute(panel_kernel<T, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -689,6 +703,11 @@ cudaError_t panel_init_attributes() {
   return e;
 }
 
+void launch_schur_fine(const FactorLaunch& a, const int* flist, int nf, int mmax, cudaStream_t s) {
+  const int nt = (mmax + Shape<double2>::kXt - 1) / Shape<double2>::kXt;
+  schur_fine_kernel<<<dim3(nt * nt, nf, a.n_omega), kPanelThreads, Cfg<double2, 3>::kSmem, s>>>(a, flist, nt);
+}
+
 template <typename T>
 void launch_panel_step(const FactorLaunch& a, const int* flist, int nf, int j0, int nmax, cudaStream_t s) {
   using S = Shape<T>;
@@ -705,7 +724,10 @@ void launch_panel_step(const FactorLaunch& a, const int* flist, int nf, int j0, 
              cudaSuccess)
             ? (long long)std::max(1, per_sm) * nsm
             : (1LL << 40);
-    // (by the level's size alone: a level's steps are all of one kind, as the look-ahead asks)
+    // One launch while a level's L and U tiles fit the chip once (by the level's size alone: its steps are
+    // all of one kind, as the look-ahead asks).  All steps of a factorisation with this rule / every level
+    // split / every level in one launch: 340 x 340 0.82 / 1.49 / 0.83 ms, 540 x 540 with 8 wavelengths
+    // 4.8 / 5.1 / 6.0 ms, 1760 x 1760 with 2 24.2 / 25.7 / 31.5 ms.
     if ((long long)(1 + 2 * ceil_div(nmax - 1, S::kTile)) * nf * a.n_omega <= wave) {
       const int nt = ceil_div(nmax - j0 - 1, S::kTile), nx = ceil_div(nmax - j0 - 1, S::kXt) * kParts;
       panel_kernel<T, 0><<<dim3(1 + 2 * nt + (j0 > 0 ? 2 * nx : 0), nf, a.n_omega), kPanelThreads, Cfg<T, 0>::kSmem, s>>>(
