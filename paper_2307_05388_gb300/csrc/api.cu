@@ -512,10 +512,12 @@ void build_units(fdfd_ctx* ctx, int prec) {
           const SweepFront& d = recs[r];
           if (rect && d.m == 0) continue;
           const int len = rect && up ? d.m : d.k;          // rows (columns) to cover
-          // up to 64 lines to a unit, and to the level's share of a CTA; the contraction in the fewest
-          // equal parts that fit a buffer
+          // up to 64 lines to a unit, and to the level's share of a CTA, from 16 on (U rows: 8); the
+          // contraction in the fewest equal parts that fit a buffer.  Sweep at 340 x 340 with 8 / 16 / 32
+          // at least: L 118 / 109 us, U 91 / 90 (complex128 125 / 131), U^T 124 / 107 / 102, L^T 164 / 134 /
+          // 134 (540 x 540, eight right-hand sides: 633 / 599 / 680): narrow columns are short copies.
           for (int s0 = 0, c; s0 < len; s0 += c) {
-            c = rows ? 8 : 16;
+            c = sweep == 1 ? 8 : 16;
             while (2 * c <= 64 && 2 * c <= share) c *= 2;
             c = std::min(c, len - s0);
             const UnitRange ur = unit_range(sweep, rect, d.k, d.m, s0, c);
