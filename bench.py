@@ -269,7 +269,7 @@ def main():
     ap.add_argument("--gmres-restart", type=int, default=0,
                     help="Krylov vectors per FGMRES cycle (0: the library default, 8)")
     ap.add_argument("--rhs-pairs", type=int, default=0, choices=[0, 1],
-                    help="sweeps take a wavelength's right-hand sides two at a time (1) or one at a time (0, default)")
+                    help="accepted, without effect: sweeps always take a wavelength's right-hand sides two at a time")
     ap.add_argument("--optimizer", default="workload", choices=["workload", "sign", "adam"],
                     help="the design update between iterations (not timed): the workload's own (default; "
                          "Adam at lr 0.01 for c4, a sign step for the others), or the one named")
