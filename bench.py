@@ -49,9 +49,9 @@ L2_FLUSH_BYTES = 512 << 20
 FP32_LANES_PER_SM = 128
 FP64_FMA_PER_SM = 2       # FP64 FMAs per SM per clock on this part (ncu dfma peak_sustained)
 # DRAM bytes (read + write) of one sweep launch over its algorithmic bytes, from the ncu capture of
-# a C4 one-wavelength L sweep (profiles/flow_sweep_c4_one_wavelength.md: 927.9 + 99.3 MB against
-# 559.8 MB of L11^-1 and L21 entries); a full launch's traffic is scaled from it by its algorithmic bytes
-SWEEP_TRAFFIC_RATIO = (927.9 + 99.3) / 559.8
+# a C4 one-wavelength L sweep (profiles/flow_sweep_c4_one_wavelength.md: 701.4 + 32.1 MB against
+# 580.2 MB of L11^-1 and L21 entries); a full launch's traffic is scaled from it by its algorithmic bytes
+SWEEP_TRAFFIC_RATIO = (701.4 + 32.1) / 580.2
 DATA = "synthetic (seeded design density and guide; the paper's devices are not published)"
 DTYPE = "c64 factors + c128 refinement"
 
@@ -480,7 +480,7 @@ def main():
                     "traffic": per_launch_bytes * SWEEP_TRAFFIC_RATIO,
                     "traffic_unit": "bytes per launch",
                     "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of a C4 one-wavelength L "
-                                      "sweep (1.027 GB against 0.560 GB algorithmic), scaled to this launch by its "
+                                      "sweep (0.734 GB against 0.580 GB algorithmic), scaled to this launch by its "
                                       "algorithmic bytes",
                     "algorithmic_bytes_per_launch": per_launch_bytes,
                     "peak_source": f"{pk['src']} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}
