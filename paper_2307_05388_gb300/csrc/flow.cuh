@@ -386,10 +386,11 @@ __device__ __forceinline__ void block_rows(const T* __restrict__ A, int stride, 
 // out(j, sum_{r in [lo(j), hi(j))} A[r][j] vec[r]) for columns j < ncols (rows < nrows): lanes over
 // 16 or 32 columns, the rows split over the rest of the CTA; partial sums through red in a fixed
 // order.  Contains barriers of the
-// working warps.
+// working warps (none without columns).
 template <int TH, typename T, int NR, int UN, typename Lo, typename Hi, typename Out>
 __device__ __forceinline__ void block_cols(const T* __restrict__ A, int stride, int ncols, int nrows, const T* vec,
                                            Lo lo, Hi hi, Out out, T* red) {
+  if (ncols <= 0) return;
   const int CW = ncols <= 16 ? 16 : 32;                // columns of a group
   const int tid = threadIdx.x;
   const int cl = tid & (CW - 1), part = tid / CW, parts = TH / CW;

@@ -79,7 +79,8 @@ FDFD_HD inline UnitRange unit_range(int sweep, bool rect, int k, int m, int r0, 
 
 // A block staged row by row: rows [row0, row0 + rows) and columns [col0, col0 + cols) of the
 // inverse block (tri) or of the front (rect), in shared memory at a row stride of `stride`
-// elements; the first wanted column is `shift` elements in (rows start on 16 bytes).
+// elements; the first wanted column is `shift` elements in (rows start on 16 bytes).  An empty block
+// (the off-diagonal block of a front without boundary rows) has no rows: nothing is copied.
 struct StageGeom {
   int row0, rows, col0, cols, stride, shift;
 };
@@ -88,7 +89,8 @@ struct StageGeom {
 // th: working threads of the CTA.
 FDFD_HD inline StageGeom stage_geom(int es, int sweep, bool rect, int k, int ld, int ldk, int r0, int cnt, int a, int b,
                                     int th) {
-  StageGeom s;
+  StageGeom s{};
+  if (cnt <= 0 || b <= a) return s;
   const int odd = es == 8 ? 1 : 0;             // alignment of a row's start and length: 2 entries of 8 bytes
   const int lim = rect ? ld : ldk;             // entries a row holds, a multiple of 4
   int c0, c1;                                  // wanted columns [c0, c1)
