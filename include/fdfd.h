@@ -358,6 +358,16 @@ fdfd_status fdfd_selftest_wait(fdfd_ctx* ctx);
  * the context stays usable.  Any other status is a failure. */
 fdfd_status fdfd_selftest_mbar_wait(fdfd_ctx* ctx);
 
+/* The sweeps' own way out: one raw sweep pair on the cached factors (zero right-hand
+ * sides) in which sweep `sweep` (0 L, 1 U, 2 U^T, 3 L^T; the symmetric form has 0 and
+ * 3) asks more of front f than it will ever complete.  Whatever depends on f gives up after
+ * its bounded polls, the CTAs run their staged units to the end and leave, and the call
+ * (synchronised, about a second) returns FDFD_ERR_TIMEOUT; FDFD_OK when nothing waits for
+ * f in that sweep (the last front of an order).  The counts are put back, the error word is cleared
+ * and the context stays usable.  FDFD_ERR_ARG: no such front or sweep; FDFD_ERR_STATE: no
+ * cached factorisation. */
+fdfd_status fdfd_selftest_sweep(fdfd_ctx* ctx, int sweep, int f);
+
 /* The same bounded wait as fdfd_selftest_wait, left for the caller to find: the
  * probe kernel and the copy of the error word back to the host are queued on the
  * context's stream and the call returns FDFD_OK without synchronising.  Once the

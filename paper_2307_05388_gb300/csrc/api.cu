@@ -2201,6 +2201,48 @@ fdfd_status fdfd_selftest_wait(fdfd_ctx* ctx) {
   return check_flow_err(ctx);
 }
 
+fdfd_status fdfd_selftest_sweep(fdfd_ctx* ctx, int sweep, int f) {
+  if (!ctx || sweep < 0 || sweep > 3 || f < 0) return FDFD_ERR_ARG;
+  ctx->err.clear();
+  if (!ctx->uploaded || !(ctx->valid32 || ctx->valid64) || ctx->opt.mode == FDFD_MODE_PLAIN)
+    return fail(ctx, FDFD_ERR_STATE, "fdfd_selftest_sweep needs a cached factorisation (fdfd_factor first)");
+  const int prec = ctx->valid64 ? 1 : 0;
+  const size_t nf = ctx->plan.fronts.size();
+  const bool sym = prec == 0 && ctx->sym32;
+  if ((size_t)f >= nf || (sym && (sweep == 1 || sweep == 2))) return fail(ctx, FDFD_ERR_ARG, "no such front or sweep");
+  CKS(check_flow_err(ctx));
+  CKS(ensure_ws(ctx, 1));
+  const size_t bytes = sizeof(double2) * ctx->n_omega * (size_t)n_cells(ctx);
+  double2* v = nullptr;
+  CK(dalloc(&v, 2 * bytes));
+  // the front's two counts of this sweep (all its units, its phase-1 units), out of reach
+  const int far = 1 << 30;
+  int* need = ctx->d_need[prec] + 2 * (size_t)sweep * nf + f;
+  const int* host = ctx->h_need[prec].data() + 2 * (size_t)sweep * nf + f;
+  cudaStream_t s = ctx->stream;
+  cudaError_t e = cudaMemsetAsync(v, 0, 2 * bytes, s);
+  for (size_t i = 0; i < 2 && e == cudaSuccess; ++i)
+    e = cudaMemcpyAsync(need + i * nf, &far, sizeof(int), cudaMemcpyHostToDevice, s);
+  fdfd_status st = FDFD_OK;
+  if (e == cudaSuccess) {
+    const int transpose = sweep >= 2 && !sym;
+    double2* x = v + bytes / sizeof(double2);
+    st = prec ? sweeps<double2>(ctx, 1, transpose, v, x) : sweeps<float2>(ctx, 1, transpose, v, x);
+  }
+  cudaError_t e2 = cudaSuccess;
+  for (size_t i = 0; i < 2 && e2 == cudaSuccess; ++i)
+    e2 = cudaMemcpyAsync(need + i * nf, host + i * nf, sizeof(int), cudaMemcpyHostToDevice, s);
+  if (e2 == cudaSuccess)
+    e2 = cudaMemcpyAsync(ctx->h_flow_err, ctx->d_flow_err, sizeof(int), cudaMemcpyDeviceToHost, s);
+  const cudaError_t e3 = cudaStreamSynchronize(s);
+  cudaFree(v);
+  CKS(st);
+  CK(e);
+  CK(e2);
+  CK(e3);
+  return check_flow_err(ctx);
+}
+
 fdfd_status fdfd_selftest_mbar_wait(fdfd_ctx* ctx) {
   if (!ctx) return FDFD_ERR_ARG;
   ctx->err.clear();

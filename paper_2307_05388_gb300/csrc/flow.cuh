@@ -52,11 +52,53 @@ namespace fdfd {
 namespace {
 
 // A CTA: TH working threads, the producer warp and the publishing warp.
-constexpr unsigned long long kFullWaitNs = 8000000000ull;   // working warps wait for a staged unit: outlasts the
-constexpr unsigned long long kFreeWaitNs = 6000000000ull;   // producer's wait for a buffer and every dependency wait
+// Limits of the waits, each longer than what it waits for may take: the producer's for a buffer (longer than
+// every dependency wait), the publisher's for a finished unit, the working warps' for a staged one (the
+// publisher ends that one first, staged_wait).
+constexpr unsigned long long kFreeWaitNs = 6000000000ull;
+constexpr unsigned long long kDoneWaitNs = 16000000000ull;
+constexpr unsigned long long kStagedWaitNs = 32000000000ull;
 
 // barrier of the working warps
 template <int TH> __device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TH) : "memory"); }
+
+// mbar_wait with one answer for the whole warp: each lane's own limit may pass at another poll, and lanes
+// that part here would meet different warp operations.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
+
+// Whether the CTA goes on: one word, written by the publisher alone.  The working warps share named barriers,
+// so either all of them run a unit or none.  They do not time out on their own: when a unit is overdue the
+// publisher asks, looks whether it is staged after all, and then says so once.  A warp that found the unit
+// staged before the question is seen by that look; one that finds it staged later reads the question
+// and waits for the answer.
+enum StopWord { kGoOn = 0, kStopAsked = 1, kStopped = 2 };
+
+// Working warps: the unit is staged and the CTA goes on.  (The limit alone ends it for a unit that no
+// producer will stage any more; then every warp's does.)
+__device__ __forceinline__ bool staged_wait(uint32_t bar, uint32_t parity, const volatile int* stop) {
+  unsigned long long t0 = 0;
+  for (uint32_t it = 0; it < (1u << 28); ++it) {
+    const bool in = mbar_try(bar, parity);
+    const int word = *stop;
+    if (in && word == kGoOn) return true;
+    if (word == kStopped) return false;
+    if ((it & 63) == 63) {
+      const unsigned long long now = gtimer();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > kStagedWaitNs) return false;
+    }
+  }
+  return false;
+}
+
+// The publisher (one lane): the unit behind `bar` is overdue.
+__device__ __forceinline__ void stop_unless_staged(uint32_t bar, uint32_t parity, volatile int* stop) {
+  *stop = kStopAsked;
+  asm volatile("fence.sc.cta;" ::: "memory");
+  *stop = mbar_try(bar, parity) ? kGoOn : kStopped;
+}
 
 // Vector entries written by other CTAs of the same launch (the dataflow sweep)
 // are read through L2 only: the per-SM L1 is not coherent.
@@ -443,10 +485,12 @@ __device__ __forceinline__ void block_cols(const T* __restrict__ A, int stride, 
 //              off-diagonal units of a front wait for its inverse-block units;
 //   top-down:  whole-front / off-diagonal units wait for the parent; the
 //              inverse-block units of a front wait for its off-diagonal units.
-// Every wait gives up after kSpinLimit polls: it sets *err and the CTA's abort
+// Every dependency wait gives up after kSpinLimit polls: it sets *err and the CTA's abort
 // word; the CTA's producer then takes no more units, its working warps run the
 // one or two staged units to the end (nothing of them is published) and the CTA
-// leaves once its copies have landed.
+// leaves once its copies have landed.  The waits inside a CTA have limits of their own, and
+// what follows one is decided for a whole warp, or for all working warps, at once
+// (warp_wait, staged_wait).
 // ---------------------------------------------------------------------------
 constexpr int kSpinLimit = 1 << 21;
 
@@ -851,7 +895,7 @@ __device__ __forceinline__ void prefetch_vectors(const SolveLaunch& a, const Flo
                                                  const double2* __restrict__ in) {
   constexpr bool kUp = SWEEP == 0 || SWEEP == 2;
   const int lane = threadIdx.x & 31;
-  if (!mbar_wait(full, parity, kFreeWaitNs)) return;
+  if (!warp_wait(full, parity, kFreeWaitNs)) return;
   const int cnt = (un.kind >> 8) & 0xff;
   for (int j = 0; j < cnt; ++j) {
     const SweepFront& d = *reinterpret_cast<const SweepFront*>(buf + 16 * (size_t)un.off[j]);
@@ -885,7 +929,7 @@ flow_kernel(SolveLaunch a, FlowQueue q, const double2* __restrict__ in, double2*
   __shared__ __align__(8) uint64_t bars[6];
   __shared__ __align__(16) SweepUnit s_unit[2];
   __shared__ int s_wl[2], s_ok[2];
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_stop;
   const int nf = q.n_fronts;
   int* head = q.ctr;
   int* done0 = q.ctr + 1;                       // [n_omega launched][nf]
@@ -900,6 +944,7 @@ flow_kernel(SolveLaunch a, FlowQueue q, const double2* __restrict__ in, double2*
     }
     mbar_init_fence();
     s_abort = 0;
+    s_stop = kGoOn;
   }
   __syncthreads();
   if (warp == TH / 32) {
@@ -913,6 +958,8 @@ flow_kernel(SolveLaunch a, FlowQueue q, const double2* __restrict__ in, double2*
       if (lane == 0 && *(volatile int*)&s_abort == 0) v = atomicAdd(head, 1);
       return __shfl_sync(0xffffffffu, v, 0);
     };
+    // the working warps may set it at any time: one lane reads it for all
+    auto aborted = [&]() { return __shfl_sync(0xffffffffu, *(volatile int*)&s_abort, 0) != 0; };
     int u = take();
     SweepUnit un{};
     if (u < total) un = q.units[u / a.n_omega];
@@ -923,12 +970,12 @@ flow_kernel(SolveLaunch a, FlowQueue q, const double2* __restrict__ in, double2*
         prefetch_vectors<T, SWEEP>(a, q, s_unit[b ^ 1], s_wl[b ^ 1] + a.w0, smem + (size_t)(b ^ 1) * bufsz,
                                    full0 + 8 * (b ^ 1), ((it - 1) >> 1) & 1, in);
       prev_packed = false;
-      if (it > two && !mbar_wait(free0 + 8 * b, ((it >> two) - 1) & 1, kFreeWaitNs)) {
+      if (it > two && !warp_wait(free0 + 8 * b, ((it >> two) - 1) & 1, kFreeWaitNs)) {
         if (lane == 0) { s_abort = 1; atomicExch(q.err, 1); }
         gave_up = true;
         break;
       }
-      if (u >= total || (un.part == 0 && *(volatile int*)&s_abort != 0)) {
+      if (u >= total || (un.part == 0 && aborted())) {
         if (lane == 0) {
           s_unit[b].kind = kUnitEnd;
           mbar_arrive(full0 + 8 * b);
@@ -999,7 +1046,14 @@ flow_kernel(SolveLaunch a, FlowQueue q, const double2* __restrict__ in, double2*
     // fronts' counters go up, after a fence that orders the CTA's stores before them ----
     for (int it = 0;; ++it) {
       const int b = it & two;
-      if (!mbar_wait(done_b0 + 8 * b, (it >> two) & 1, 2 * kFullWaitNs)) break;
+      if (!warp_wait(done_b0 + 8 * b, (it >> two) & 1, kDoneWaitNs)) {
+        if (lane == 0) {
+          s_abort = 1;
+          atomicExch(q.err, 1);
+          stop_unless_staged(full0 + 8 * b, (it >> two) & 1, &s_stop);
+        }
+        break;
+      }
       const int kc = s_unit[b].kind, kind = kc & 0xff;
       if (kind == kUnitEnd) break;
       const unsigned char* buf = smem + (size_t)b * bufsz;
@@ -1023,7 +1077,9 @@ flow_kernel(SolveLaunch a, FlowQueue q, const double2* __restrict__ in, double2*
     for (int it = 0;; ++it) {
       const int b = it & two;
       unsigned char* buf = smem + (size_t)b * bufsz;
-      if (!mbar_wait(full0 + 8 * b, (it >> two) & 1, kFullWaitNs)) {
+      const bool staged = staged_wait(full0 + 8 * b, (it >> two) & 1, &s_stop);
+      __syncwarp();
+      if (!staged) {
         if (lane == 0) { s_abort = 1; atomicExch(q.err, 1); }
         break;
       }

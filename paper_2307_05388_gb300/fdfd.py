@@ -28,7 +28,8 @@ EXPORTS = ["fdfd_default_options", "fdfd_create", "fdfd_analyze", "fdfd_factor",
            "fdfd_solve", "fdfd_objective", "fdfd_grad", "fdfd_apply", "fdfd_set_options", "fdfd_stats_get",
            "fdfd_plan_fronts", "fdfd_reset_counters", "fdfd_last_error", "fdfd_destroy",
            "fdfd_profile_enable", "fdfd_profile_get", "fdfd_solve_raw_noalloc", "fdfd_noalloc_scratch_bytes",
-           "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_mbar_wait", "fdfd_selftest_schur_tc", "fdfd_filter_project", "fdfd_filter_project_adjoint",
+           "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_mbar_wait", "fdfd_selftest_sweep",
+           "fdfd_selftest_schur_tc", "fdfd_filter_project", "fdfd_filter_project_adjoint",
            "fdfd_slab_modes", "fdfd_objective_target", "fdfd_design_iteration", "fdfd_density_eps", "fdfd_front_copy",
            "fdfd_plan_sizes"]
 HOST_EPS, HOST_OUT = 1, 2
@@ -108,6 +109,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
     lib.fdfd_selftest_wait.argtypes = [vp]
     lib.fdfd_selftest_wait_async.argtypes = [vp]
     lib.fdfd_selftest_mbar_wait.argtypes = [vp]
+    lib.fdfd_selftest_sweep.argtypes = [vp, i, i]
     lib.fdfd_slab_modes.argtypes = [i, d, vp, i, vp, vp, vp]
     lib.fdfd_last_error.argtypes = [vp]
     lib.fdfd_last_error.restype = C.c_char_p
@@ -117,7 +119,8 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
                  "fdfd_objective", "fdfd_grad", "fdfd_apply", "fdfd_set_options", "fdfd_stats_get",
                  "fdfd_plan_fronts", "fdfd_profile_enable", "fdfd_profile_get", "fdfd_filter_project",
                  "fdfd_filter_project_adjoint", "fdfd_objective_target", "fdfd_design_iteration",
-                 "fdfd_density_eps", "fdfd_front_copy", "fdfd_plan_sizes", "fdfd_selftest_mbar_wait", "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_schur_tc", "fdfd_slab_modes"):
+                 "fdfd_density_eps", "fdfd_front_copy", "fdfd_plan_sizes", "fdfd_selftest_mbar_wait", "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_sweep",
+                 "fdfd_selftest_schur_tc", "fdfd_slab_modes"):
         getattr(lib, name).restype = C.c_int
     return lib
 
@@ -368,6 +371,11 @@ class Solver:
         """Runs the tensor-core pipeline's bounded mbarrier wait on a barrier nothing arrives at;
         returns the status (7 = gave up as designed)."""
         return int(_lib.fdfd_selftest_mbar_wait(self._h))
+
+    def selftest_sweep(self, sweep: int, f: int) -> int:
+        """One raw sweep pair in which sweep `sweep` (0 L, 1 U, 2 U^T, 3 L^T) waits for front f in vain;
+        returns the status (7 = gave up as designed, 0 = nothing waits for f)."""
+        return int(_lib.fdfd_selftest_sweep(self._h, int(sweep), int(f)))
 
     def selftest_wait_async(self) -> int:
         """Queues the same wait without synchronising; the next call that checks the error word
