@@ -427,9 +427,9 @@ __device__ __forceinline__ void block_rows(const T* __restrict__ A, int stride, 
 
 // out(j, sum_{r in [lo(j), hi(j))} A[r][j] vec[r]) for columns j < ncols (rows < nrows): lanes over
 // 16 or 32 columns, the rows split over the rest of the CTA; partial sums through red in a fixed
-// order.  Contains barriers of the
+// order.  ORDERED: a thread adds its rows one to the next, else in two sums in turn.  Contains barriers of the
 // working warps (none without columns).
-template <int TH, typename T, int NR, int UN, typename Lo, typename Hi, typename Out>
+template <int TH, typename T, int NR, int UN, bool ORDERED = false, typename Lo, typename Hi, typename Out>
 __device__ __forceinline__ void block_cols(const T* __restrict__ A, int stride, int ncols, int nrows, const T* vec,
                                            Lo lo, Hi hi, Out out, T* red) {
   if (ncols <= 0) return;
@@ -452,7 +452,7 @@ __device__ __forceinline__ void block_cols(const T* __restrict__ A, int stride, 
 #pragma unroll
         for (int u = 0; u < UN; ++u) f[u] = A[(size_t)(r + u) * stride + j];
 #pragma unroll
-        for (int u = 0; u < UN; ++u) vfma(f[u], vget<T, NR>(vec, r + u), (u & 1) ? a1 : a0);
+        for (int u = 0; u < UN; ++u) vfma(f[u], vget<T, NR>(vec, r + u), (u & 1) && !ORDERED ? a1 : a0);
       }
       for (; r < re; ++r) vfma(A[(size_t)r * stride + j], vget<T, NR>(vec, r), a0);
     }
@@ -748,10 +748,17 @@ __device__ __forceinline__ bool whole_front(const SolveLaunch& a, const FlowQueu
       else
         block_cols<TH, T, NR, 4>(B, bs, k, m, v + k * NR, [](int) { return 0; }, [&](int) { return m; }, put, red);
       work_sync<TH>();
-      block_tri<TH, T, SWEEP, NR, PACKED>(X, k, ldk, ws, [&](int i, const Vals<T, NR>& s) {
+      auto put_k = [&](int i, const Vals<T, NR>& s) {
         if (SWEEP == 1) put_x<T, SWEEP, NR>(a, c, cells[i], w, s);
         else put_x<T, SWEEP, NR>(a, c, cells[Pm[i]], w, vadd(vget<T, NR>(ws, i), s));
-      });
+      };
+      // L^T of a dense front: neighbouring rows one after the other in one thread's sum.  Where the symmetric form
+      // meets a small pivot its row and the next have large entries that cancel; in sums that take rows in turn
+      // every term between is rounded at that size (540 x 540, growth 2e4: 2 to 3 times the residual in
+      // nine directions, and FGMRES took 12 to 14 vectors instead of 9).  complex128 factors always have pivots.
+      if constexpr (SWEEP == 3 && !PACKED && es == 8)
+        block_cols<TH, T, NR, 4, true>(X, ldk, k, k, ws, [](int j) { return j + 1; }, [&](int) { return k; }, put_k, red);
+      else block_tri<TH, T, SWEEP, NR, PACKED>(X, k, ldk, ws, put_k);
     }
     if (rc + NR < a.r0 + a.nr) work_sync<TH>();
   }
