@@ -47,7 +47,15 @@ template <typename P>
 cudaError_t dalloc(P** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
-  return cudaMalloc((void**)p, bytes);
+  const cudaError_t e = cudaMalloc((void**)p, bytes);
+  if (e != cudaSuccess) (void)cudaGetLastError();   // reported here; the next launch's check is not about it
+  return e;
+}
+// The same for a buffer that is kept: one that an earlier call, which failed on the way, left out is
+// allocated now.
+template <typename P>
+cudaError_t dneed(P** p, size_t bytes) {
+  return *p ? cudaSuccess : dalloc(p, bytes);
 }
 
 }  // namespace
@@ -551,6 +559,7 @@ fdfd_status upload(fdfd_ctx* ctx, P** dst, const std::vector<P>& v);
 fdfd_status ensure_units(fdfd_ctx* ctx, int prec) {
   if (ctx->d_units[prec]) return FDFD_OK;
   build_units(ctx, prec);
+  free_ptr(ctx->d_need[prec]);                      // (left by a call whose second upload failed)
   CKS(upload(ctx, &ctx->d_need[prec], ctx->h_need[prec]));
   return upload(ctx, &ctx->d_units[prec], ctx->h_units[prec]);
 }
@@ -777,25 +786,26 @@ fdfd_status upload_plan(fdfd_ctx* ctx) {
 // Device runtime: kernel attributes, stencil coefficient tables, eps buffer.
 fdfd_status ensure_runtime(fdfd_ctx* ctx) {
   if (ctx->device < 0) {
-    CK(cudaGetDevice(&ctx->device));
+    int dev = -1;
+    CK(cudaGetDevice(&dev));
     CK(factor_init_attributes());
     CK(panel_init_attributes());
     CK(tc_init_attributes());
     CK(solve_init_attributes());
-    CK(dalloc(&ctx->d_cxm, sizeof(double2) * ctx->n_omega * ctx->nx));
-    CK(dalloc(&ctx->d_cxp, sizeof(double2) * ctx->n_omega * ctx->nx));
-    CK(dalloc(&ctx->d_cym, sizeof(double2) * ctx->n_omega * ctx->ny));
-    CK(dalloc(&ctx->d_cyp, sizeof(double2) * ctx->n_omega * ctx->ny));
-    CK(dalloc(&ctx->d_sxc, sizeof(double2) * ctx->n_omega * ctx->nx));
-    CK(dalloc(&ctx->d_syc, sizeof(double2) * ctx->n_omega * ctx->ny));
-    CK(dalloc(&ctx->d_k0dx, sizeof(double) * ctx->n_omega));
-    CK(dalloc(&ctx->d_k0dx2, sizeof(double) * ctx->n_omega));
-    CK(dalloc(&ctx->d_eps, sizeof(double) * n_cells(ctx)));
-    CK(dalloc(&ctx->d_growth_max, sizeof(float)));
-    CK(cudaMallocHost((void**)&ctx->h_growth_max, sizeof(float)));
-    CK(dalloc(&ctx->d_flow_err, sizeof(int)));
+    CK(dneed(&ctx->d_cxm, sizeof(double2) * ctx->n_omega * ctx->nx));
+    CK(dneed(&ctx->d_cxp, sizeof(double2) * ctx->n_omega * ctx->nx));
+    CK(dneed(&ctx->d_cym, sizeof(double2) * ctx->n_omega * ctx->ny));
+    CK(dneed(&ctx->d_cyp, sizeof(double2) * ctx->n_omega * ctx->ny));
+    CK(dneed(&ctx->d_sxc, sizeof(double2) * ctx->n_omega * ctx->nx));
+    CK(dneed(&ctx->d_syc, sizeof(double2) * ctx->n_omega * ctx->ny));
+    CK(dneed(&ctx->d_k0dx, sizeof(double) * ctx->n_omega));
+    CK(dneed(&ctx->d_k0dx2, sizeof(double) * ctx->n_omega));
+    CK(dneed(&ctx->d_eps, sizeof(double) * n_cells(ctx)));
+    CK(dneed(&ctx->d_growth_max, sizeof(float)));
+    if (!ctx->h_growth_max) CK(cudaMallocHost((void**)&ctx->h_growth_max, sizeof(float)));
+    CK(dneed(&ctx->d_flow_err, sizeof(int)));
     CK(cudaMemsetAsync(ctx->d_flow_err, 0, sizeof(int), ctx->stream));
-    CK(cudaMallocHost((void**)&ctx->h_flow_err, sizeof(int)));
+    if (!ctx->h_flow_err) CK(cudaMallocHost((void**)&ctx->h_flow_err, sizeof(int)));
     *ctx->h_flow_err = 0;
     CK(cudaMemcpyAsync(ctx->d_k0dx, ctx->k0dx.data(), sizeof(double) * ctx->n_omega, cudaMemcpyHostToDevice,
                        ctx->stream));
@@ -803,6 +813,7 @@ fdfd_status ensure_runtime(fdfd_ctx* ctx) {
                 ctx->d_k0dx, ctx->n_omega,
                 ctx->nx, ctx->ny, ctx->pml.npml_x, ctx->pml.npml_y, ctx->pml.ln_R, ctx->pml.order, ctx->stream);
     CK(cudaGetLastError());
+    ctx->device = dev;                                 // (once all of it is there)
   }
   return FDFD_OK;
 }
@@ -836,23 +847,22 @@ fdfd_status ensure_store(fdfd_ctx* ctx, int prec) {
   const Plan& p = ctx->plan;
   CKS(ensure_units(ctx, prec));
   const size_t nfr = p.fronts.size();
-  if (!ctx->d_growth) CK(dalloc(&ctx->d_growth, sizeof(float) * nfr * ctx->n_omega));
-  if (!ctx->d_swp)
-    CK(dalloc(&ctx->d_swp, sizeof(int) * (size_t)kSwapScratchInts * std::max(1, ctx->max_nlarge) * ctx->n_omega));
-  if (!ctx->d_dblk)
-    CK(dalloc(reinterpret_cast<char**>(&ctx->d_dblk),
-              sizeof(double2) * (size_t)kDiagBlkElems * std::max(1, ctx->max_nlarge) * ctx->n_omega));
-  if (prec == 0 && !ctx->d_store32) {
-    CK(dalloc(&ctx->d_store32, sizeof(float2) * (size_t)p.store_total * ctx->n_omega));
-    CK(dalloc(&ctx->d_perm32, sizeof(int) * (size_t)std::max(1, p.perm_total) * ctx->n_omega));
-    CK(dalloc(&ctx->d_inv32, sizeof(float2) * (size_t)p.inv_total * ctx->n_omega));
-    CK(dalloc(&ctx->d_pack32, sizeof(float2) * (size_t)std::max<long long>(2, 2 * p.pack_total) * ctx->n_omega));
-  }
-  if (prec == 1 && !ctx->d_store64) {
-    CK(dalloc(&ctx->d_store64, sizeof(double2) * (size_t)p.store_total * ctx->n_omega));
-    CK(dalloc(&ctx->d_perm64, sizeof(int) * (size_t)std::max(1, p.perm_total) * ctx->n_omega));
-    CK(dalloc(&ctx->d_inv64, sizeof(double2) * (size_t)p.inv_total * ctx->n_omega));
-    CK(dalloc(&ctx->d_pack64, sizeof(double2) * (size_t)std::max<long long>(2, 2 * p.pack_total) * ctx->n_omega));
+  const size_t nw = ctx->n_omega, large = std::max(1, ctx->max_nlarge);
+  const size_t store = (size_t)p.store_total * nw, perm = (size_t)std::max(1, p.perm_total) * nw,
+               inv = (size_t)p.inv_total * nw, pack = (size_t)std::max<long long>(2, 2 * p.pack_total) * nw;
+  CK(dneed(&ctx->d_growth, sizeof(float) * nfr * nw));
+  CK(dneed(&ctx->d_swp, sizeof(int) * kSwapScratchInts * large * nw));
+  CK(dneed(reinterpret_cast<char**>(&ctx->d_dblk), sizeof(double2) * kDiagBlkElems * large * nw));
+  if (prec == 0) {
+    CK(dneed(&ctx->d_store32, sizeof(float2) * store));
+    CK(dneed(&ctx->d_perm32, sizeof(int) * perm));
+    CK(dneed(&ctx->d_inv32, sizeof(float2) * inv));
+    CK(dneed(&ctx->d_pack32, sizeof(float2) * pack));
+  } else {
+    CK(dneed(&ctx->d_store64, sizeof(double2) * store));
+    CK(dneed(&ctx->d_perm64, sizeof(int) * perm));
+    CK(dneed(&ctx->d_inv64, sizeof(double2) * inv));
+    CK(dneed(&ctx->d_pack64, sizeof(double2) * pack));
   }
   return FDFD_OK;
 }
@@ -1707,6 +1717,8 @@ fdfd_status fdfd_solve(fdfd_ctx* ctx, const double* b_dev, double* x_dev, int nr
   if (!ctx || !b_dev || !x_dev || nrhs <= 0 || b_dev == x_dev) return FDFD_ERR_ARG;
   ctx->err.clear();
   if (!ctx->have_eps) return fail(ctx, FDFD_ERR_STATE, "fdfd_solve before fdfd_factor");
+  if (ctx->opt.mode != FDFD_MODE_PLAIN && !ctx->valid32 && !ctx->valid64)
+    return fail(ctx, FDFD_ERR_STATE, "no cached factorisation (the last fdfd_factor failed)");
   bool handled = false;
   const fdfd_status st = solve_direct(ctx, b_dev, x_dev, nrhs, transpose, &handled);
   if (handled) {
@@ -1844,11 +1856,9 @@ fdfd_status fdfd_design_iteration(fdfd_ctx* ctx, const double* eps_design, const
     CK(dalloc(&ctx->d_ito, sizeof(double2) * S));
     ctx->it_nrhs = nrhs;
   }
-  if (!ctx->d_itF) {
-    CK(dalloc(&ctx->d_itF, sizeof(double)));
-    CK(dalloc(&ctx->d_itg, sizeof(double) * nd));
-    CK(dalloc(&ctx->d_itepsd, sizeof(double) * nd));
-  }
+  CK(dneed(&ctx->d_itF, sizeof(double)));
+  CK(dneed(&ctx->d_itg, sizeof(double) * nd));
+  CK(dneed(&ctx->d_itepsd, sizeof(double) * nd));
   const double* epsd = eps_design;
   if (flags & FDFD_HOST_EPS) {
     CK(cudaMemcpyAsync(ctx->d_itepsd, eps_design, sizeof(double) * nd, cudaMemcpyHostToDevice, ctx->stream));
@@ -1909,6 +1919,7 @@ static fdfd_status ensure_taps(fdfd_ctx* ctx, double radius) {
   free_ptr(ctx->d_tapw);
   ctx->d_taps = nullptr;
   ctx->d_tapw = nullptr;
+  ctx->tap_radius = 0;                      // until the new ones are there
   CK(dalloc(&ctx->d_taps, sizeof(int2) * off.size()));
   CK(dalloc(&ctx->d_tapw, sizeof(double) * wt.size()));
   CK(cudaMemcpy(ctx->d_taps, off.data(), sizeof(int2) * off.size(), cudaMemcpyHostToDevice));
