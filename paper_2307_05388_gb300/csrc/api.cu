@@ -181,7 +181,8 @@ struct fdfd_ctx {
   unsigned char* d_stat = nullptr;
   unsigned char* h_stat = nullptr;  // pinned
   size_t stat_bytes = 0;
-  bool gm_second[2] = {false, false};   // the next solve runs the second projection [transpose]
+  // the next solve launches the second projection [transpose]; belongs to the factors: forget_second()
+  bool gm_second[2] = {false, false};
 
   // per-kernel profile (CUDA events around every launch when enabled)
   bool prof_on = false;
@@ -1393,6 +1394,9 @@ fdfd_status any_active(fdfd_ctx* ctx, int S, bool inside, bool* any, double* max
   return FDFD_OK;
 }
 
+// Whether solves need the second projection is learnt from solves on the same preconditioner.
+void forget_second(fdfd_ctx* ctx) { ctx->gm_second[0] = ctx->gm_second[1] = false; }
+
 // Flexible GMRES, right-preconditioned by the cached LU, FP64 residuals and updates.
 fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int transpose) {
   const int m = std::max(1, std::min(ctx->opt.gmres_restart, multidot_max_vectors() - 1));
@@ -1405,6 +1409,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
   const int tr = transpose ? 1 : 0;
   cudaStream_t s = ctx->stream;
   const GmStat ds = gm_stat(ctx->d_stat, S), hs = gm_stat(ctx->h_stat, S);
+  auto wanted_second = [&]() { return std::any_of(hs.reorth, hs.reorth + S, [](int r) { return r != 0; }); };
   ArnoldiStep as;
   as.C = dev_coef(ctx); as.nrhs = nrhs; as.transpose = transpose;
   as.b = b; as.z = x; as.V = ctx->d_V; as.vstride = (long long)vs; as.nv = 0; as.w = ctx->d_r;
@@ -1433,6 +1438,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
     // yet; later cycles start from the true FP64 residual and decide.
     if (cycle > 0) {
       CKS(any_active(ctx, S, false, &any, &res));
+      if (wanted_second()) as.second = 1;
       if (!any) { converged = res <= tol; break; }   // a NaN residual is never converged
     }
     if (total >= ctx->opt.ir_max_iter) {
@@ -1467,6 +1473,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
       if (cycle == 0 && total == ctx->gm_expect[tr] && total < ctx->opt.ir_max_iter) break;
       if (total >= ctx->gm_expect[tr] || j + 1 == m || total >= ctx->opt.ir_max_iter) {
         CKS(any_active(ctx, S, true, &any, &res));
+        if (wanted_second()) as.second = 1;
         if (!any) break;
       }
       if (total >= ctx->opt.ir_max_iter) break;
@@ -1493,11 +1500,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
     if (mx > 0) expect = std::min<long long>(expect, mx);
   }
   ctx->gm_expect[tr] = std::max<long long>(1, expect);
-  // the second projection runs in the next solve if a system of this one wanted it
-  if (cycles > 0) {
-    ctx->gm_second[tr] = false;
-    for (int i = 0; i < S; ++i) ctx->gm_second[tr] = ctx->gm_second[tr] || hs.reorth[i] != 0;
-  }
+  if (cycles > 0) ctx->gm_second[tr] = wanted_second();
   if (!converged)
     return fail(ctx, FDFD_ERR_NOT_CONVERGED,
                 "refinement stopped at relative residual " + std::to_string(res) + " after " +
@@ -1513,6 +1516,7 @@ fdfd_status refactor_f64(fdfd_ctx* ctx) {
   const fdfd_status fst = factor_levels<double2>(ctx, false);
   ctx->opt.pivoting = piv_saved;
   CKS(fst);
+  forget_second(ctx);
   CK(cudaStreamSynchronize(ctx->stream));
   const float g64 = *ctx->h_growth_max;
   ctx->last_growth = g64;
@@ -1554,6 +1558,7 @@ fdfd_status settle_growth(fdfd_ctx* ctx, bool* fell_back = nullptr, bool* repivo
     const fdfd_status fst = factor_levels<float2>(ctx, false);
     ctx->opt.pivoting = piv_saved;
     CKS(fst);
+    forget_second(ctx);
     CK(cudaStreamSynchronize(ctx->stream));
     CKS(check_flow_err(ctx));
     g = *ctx->h_growth_max;
@@ -1664,6 +1669,7 @@ fdfd_status fdfd_factor(fdfd_ctx* ctx, const double* eps_dev) {
   CK(cudaMemcpyAsync(ctx->d_eps, eps_dev, sizeof(double) * n_cells(ctx), cudaMemcpyDeviceToDevice, ctx->stream));
   ctx->have_eps = true;
   ctx->valid32 = ctx->valid64 = false;
+  forget_second(ctx);
   if (ctx->opt.mode == FDFD_MODE_PLAIN) return FDFD_OK;   // factorised inside every solve
   CKS(ensure_device(ctx));
   if (ctx->opt.mode == FDFD_MODE_F64) {
@@ -1986,6 +1992,7 @@ fdfd_status fdfd_set_options(fdfd_ctx* ctx, const fdfd_options* opt) {
   ctx->opt.ir_tol = opt->ir_tol;
   ctx->opt.ir_max_iter = std::max(0, opt->ir_max_iter);
   ctx->opt.gmres_restart = std::max(1, std::min(16, opt->gmres_restart));
+  forget_second(ctx);
   return FDFD_OK;
 }
 

@@ -227,7 +227,7 @@ struct ArnoldiStep {
   double2* partial;        // [arnoldi_partials(n, nsys)]
   int* cnt;                // [nsys] zero, left zero
   double2 *h1, *h2;        // projections, [nsys][multidot_max_vectors()]
-  double2 *e2, *hn;        // squared norms (x), [nsys]
+  double2 *e2, *hn;        // squared norms (x) before and after a projection, [nsys]
   int* nj;                 // Krylov vectors used in this cycle, [nsys]
   int* nj_out;             // ... in the one before, [nsys]
   int* active;
@@ -236,7 +236,7 @@ struct ArnoldiStep {
   double* vscale;
   double2 *H, *cs, *sn, *g;
   double* loss;            // orthogonality lost so far, [nsys]
-  int* reorth;             // 1: this solve needed (or wanted) a second projection, [nsys]
+  int* reorth;             // 1: a column of this solve needed the second projection, [nsys]
   int* again;              // 1: kPassProj left the column to the second projection, [nsys]
   int second;              // the second projection's passes are launched
   int m;

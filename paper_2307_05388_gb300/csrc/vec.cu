@@ -280,10 +280,11 @@ __global__ void scale_vec_kernel(double2* dst, const double2* src, const double*
 // vector that is orthogonal only to the rounding of the large component: Gram-Schmidt used to run
 // twice for that.  Taking v_j off first (h_jj = 1 + V_j^H e) removes the large component exactly, and
 // one projection of the small rest is enough unless it cancels again.  What one projection loses is
-// followed per system: loss_{j+1} = loss_j |e| / |e'| + 2^-52 / |e'|.  Where it passes 1e-3 the cycle of that
-// system ends (the next one starts from the true residual) and the host asks for the second
-// projection (kPassDots2, kPassProj2) in the next solve of that direction; it then runs where the
-// first one cancelled more than a factor of ten.
+// followed per system: loss_{j+1} = (loss_j |e| + 2^-52) / |e'|.  Where it would pass 1e-3 the second
+// projection (kPassDots2, kPassProj2) runs, after which loss_{j+1} = (loss_j + 2^-52) |e'| / |e''|.  Its two
+// launches are left out until a system has asked for it: the first time, the cycle of that system ends there
+// (the next one starts from the true residual) and the host launches them from then on, in this solve and
+// in the following ones of that direction on these factors as long as they run for some system.
 //
 // FP64 is 2 multiply-adds per clock and SM on this part and bounds these passes.  Eight entries per thread and
 // a butterfly that halves the values with the lanes (6 additions for two complex sums where a plain
@@ -432,27 +433,24 @@ arnoldi_kernel(ArnoldiStep g, int pass) {
     if (sys == 0) *g.err_out = *g.err;
   } else if (project) {
     const double2* h = g.h1 + (size_t)sys * kMaxDot;
-    const double hn2 = norm->x, en2 = g.e2[sys].x;
-    if (pass == kPassProj) {
-      const bool cancelled = hn2 < 0.01 * en2;
-      if (cancelled && g.second) {
-        g.again[sys] = 1;                 // the Givens update waits for the second projection
-        return;
-      }
-      g.again[sys] = 0;
-      finish_column(g, sys, h, nullptr, hn2);
-      const double hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
-      const double loss = hn > 0.0 ? g.loss[sys] * sqrt(en2) / hn + 2.220446049250313e-16 / hn : 0.0;
-      g.loss[sys] = loss;
-      if (loss > kMaxLoss) {
-        g.active[sys] = 0;
-        g.reorth[sys] = 1;
-      }
-    } else {
-      g.again[sys] = 0;
-      g.reorth[sys] = 1;                  // needed here: the next solve keeps the second projection
-      finish_column(g, sys, h, g.h2 + (size_t)sys * kMaxDot, hn2);
-      g.loss[sys] = 2.220446049250313e-16;
+    const double hn2 = norm->x, en2 = g.e2[sys].x;         // after and before this projection
+    const double hn = hn2 > 0.0 ? sqrt(hn2) : 0.0, en = en2 > 0.0 ? sqrt(en2) : 0.0;
+    // the rounding that the vector carries into its normalised form: of v_j's size in the first projection,
+    // of the vector's own in the second
+    const double u = 2.220446049250313e-16 * (pass == kPassProj ? 1.0 : en);
+    const double loss = hn > 0.0 ? (g.loss[sys] * en + u) / hn : 0.0;
+    if (pass == kPassProj && loss > kMaxLoss && g.second) {
+      g.again[sys] = 1;                   // the Givens update waits for the second projection
+      g.reorth[sys] = 1;
+      g.e2[sys] = make_double2(hn2, 0.0);
+      return;
+    }
+    g.again[sys] = 0;
+    finish_column(g, sys, h, pass == kPassProj ? nullptr : g.h2 + (size_t)sys * kMaxDot, hn2);
+    g.loss[sys] = loss;
+    if (loss > kMaxLoss) {
+      g.active[sys] = 0;
+      g.reorth[sys] = 1;
     }
   }
 }
