@@ -1211,8 +1211,8 @@ fdfd_status sweep_pair(fdfd_ctx* ctx, const SolveLaunch& sa, int transpose, cons
     }
     const int sweep = dir == 0 ? fwd : bwd;
     const auto& fq = ctx->flow[prec][sweep];
-    // algorithmic work: every entry of the swept triangle and of the off-diagonal block once per
-    // right-hand side, 8 flops per entry, plus the vectors
+    // algorithmic work: every entry of the swept triangle and of the off-diagonal block read once for the
+    // launch's right-hand sides, 8 flops per entry and right-hand side, and the vectors of each
     const double ent = (sweep == 0 || sweep == 3 ? ctx->ent_lower : ctx->ent_upper) + ctx->ent_rect;
     CK(cudaMemsetAsync(ctr, 0, ctr_bytes, s));
     FlowQueue q;
@@ -1227,7 +1227,7 @@ fdfd_status sweep_pair(fdfd_ctx* ctx, const SolveLaunch& sa, int transpose, cons
     q.n_fronts = (int)p.fronts.size();
     const int grid = (int)std::max<long long>(1, std::min<long long>(grid_max, (long long)fq.nu * sa.n_omega));
     static const int kinds[4] = {PK_SWEEP_L, PK_SWEEP_U, PK_SWEEP_UT, PK_SWEEP_LT};
-    Prof pr(ctx, kinds[sweep], 8.0 * ent * nsys, es * (ent + (double)p.vec_total) * nsys);
+    Prof pr(ctx, kinds[sweep], 8.0 * ent * nsys, es * (ent * sd.n_omega + (double)p.vec_total * nsys));
     launch_sweep_flow<T>(sd, sweep, q, ctx->flow_shape[prec], grid, in, out, s);
   }
   CK(cudaGetLastError());
