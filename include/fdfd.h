@@ -155,7 +155,7 @@ typedef struct {
   double growth;               /* largest |L| entry in the last factorisation */
   int n_fronts, n_levels, max_front;
   long long factor_entries;    /* stored L and U entries per wavelength */
-  long long store_bytes;       /* device bytes of front storage (all wavelengths) */
+  long long store_bytes;       /* device bytes of front storage, small fronts' packed blocks among it (all wavelengths) */
   double flops_factor;         /* full factorisation flops per wavelength (8 per complex FMA) */
   double flops_design;         /* flops of a design refactor per wavelength */
   long long repivots;          /* complex FP32 factorisations redone with partial pivoting over all

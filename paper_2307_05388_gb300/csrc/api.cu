@@ -2018,9 +2018,11 @@ fdfd_status fdfd_stats_get(fdfd_ctx* ctx, fdfd_stats* o) {
     o->factor_entries = p.factor_entries;
     o->flops_factor = p.flops_factor;
     o->flops_design = p.flops_design;
+    // (small fronts keep L21 and U12 in the packed store)
+    const long long entries = (long long)(p.store_total + 2 * p.pack_total) * ctx->n_omega;
     long long b = 0;
-    if (ctx->d_store32) b += (long long)p.store_total * ctx->n_omega * 8;
-    if (ctx->d_store64) b += (long long)p.store_total * ctx->n_omega * 16;
+    if (ctx->d_store32) b += entries * 8;
+    if (ctx->d_store64) b += entries * 16;
     o->store_bytes = b;
   }
   return FDFD_OK;

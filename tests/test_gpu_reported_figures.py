@@ -42,3 +42,12 @@ def test_sweep_bytes_count_a_factor_entry_once_a_launch(mode, es, nrhs, transpos
         assert p[name]["launches"] == groups
         assert p[name]["bytes"] == es * 2 * ((ent + rect) * groups + vec * nrhs)
         assert p[name]["flops"] == 8 * 2 * (ent + rect) * nrhs
+
+
+@pytest.mark.parametrize("mode,es", [(FD.MODE_MIXED, 8), (FD.MODE_F64, 16)])
+def test_store_bytes_cover_the_factors(mode, es):
+    """At least L21, U12 and the update matrix of every front, wherever they are kept."""
+    _, s = _solver(n_omega=3, mode=mode)
+    k, m, *_ = (v.astype(float) for v in s.plan_fronts())
+    assert s.stats()["store_bytes"] >= es * 3 * (2 * k * m + m * m).sum()
+    s.close()
