@@ -307,6 +307,13 @@ fdfd_status fdfd_plan_fronts(fdfd_ctx* ctx, int* k_host, int* m_host, int* paren
  * storage and the row stride ldk of its inverse block (host memory; NULL skips). */
 fdfd_status fdfd_plan_sizes(fdfd_ctx* ctx, int* n_host, int* ld_host, int* ldk_host);
 
+/* Sweep introspection for tests: the work units of sweep `sweep` (0 L, 1 U, 2 U^T, 3 L^T) on
+ * complex FP32 (f64 = 0) or FP64 factors, counted into counts[7] (host memory): units of small
+ * fronts a warp each, packed fronts a CTA each, other whole fronts, lines of inverse blocks, lines
+ * of off-diagonal blocks; then how many of the last two work through their contraction in several
+ * parts.  FDFD_ERR_STATE before a factorisation of that precision. */
+fdfd_status fdfd_sweep_units(fdfd_ctx* ctx, int f64, int sweep, int* counts);
+
 /* Factor introspection for tests: copies front f of wavelength w of the current
  * factorisation to host memory (synchronises the stream): front_host receives
  * n x ld entries (row-major; complex64, or complex128 if the factorisation is in

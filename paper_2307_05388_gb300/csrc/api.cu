@@ -2056,6 +2056,24 @@ fdfd_status fdfd_plan_fronts(fdfd_ctx* ctx, int* k, int* m, int* parent, int* le
   return FDFD_OK;
 }
 
+fdfd_status fdfd_sweep_units(fdfd_ctx* ctx, int f64, int sweep, int* counts) {
+  if (!ctx || !counts || sweep < 0 || sweep > 3) return FDFD_ERR_ARG;
+  const int prec = f64 ? 1 : 0;
+  if (!ctx->d_units[prec]) return fail(ctx, FDFD_ERR_STATE, "no factorisation in that precision");
+  std::fill(counts, counts + 7, 0);
+  const auto& fl = ctx->flow[prec][sweep];
+  for (int i = 0; i < fl.nu; ++i) {
+    const SweepUnit& u = ctx->h_units[prec][fl.uoff + i];
+    const int kind = u.kind & 0xff;
+    counts[kind]++;
+    if (kind < kUnitTri) continue;
+    const SweepFront& d = ctx->h_sweepf[u.rec];
+    const UnitRange r = unit_range(sweep, kind == kUnitRect, d.k, d.m, u.r0, u.cnt);
+    if (r.hi - r.lo > u.vslice) counts[kind == kUnitTri ? 5 : 6]++;
+  }
+  return FDFD_OK;
+}
+
 fdfd_status fdfd_front_copy(fdfd_ctx* ctx, int w, int f, void* front_host, void* inv_host) {
   if (!ctx || w < 0 || w >= ctx->n_omega || f < 0) return FDFD_ERR_ARG;
   ctx->err.clear();

@@ -31,7 +31,7 @@ EXPORTS = ["fdfd_default_options", "fdfd_create", "fdfd_analyze", "fdfd_factor",
            "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_mbar_wait", "fdfd_selftest_sweep",
            "fdfd_selftest_schur_tc", "fdfd_filter_project", "fdfd_filter_project_adjoint",
            "fdfd_slab_modes", "fdfd_objective_target", "fdfd_design_iteration", "fdfd_density_eps", "fdfd_front_copy",
-           "fdfd_plan_sizes"]
+           "fdfd_plan_sizes", "fdfd_sweep_units"]
 HOST_EPS, HOST_OUT = 1, 2
 
 
@@ -90,6 +90,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
     lib.fdfd_density_eps.argtypes = [vp, vp, d, d, vp]
     lib.fdfd_front_copy.argtypes = [vp, i, i, vp, vp]
     lib.fdfd_plan_sizes.argtypes = [vp, vp, vp, vp]
+    lib.fdfd_sweep_units.argtypes = [vp, i, i, vp]
     lib.fdfd_design_iteration.argtypes = [vp, vp, vp, i, vp, vp, vp, vp, vp, vp, vp, vp, i]
     lib.fdfd_apply.argtypes = [vp, vp, vp, i, i]
     lib.fdfd_set_options.argtypes = [vp, C.POINTER(Options)]
@@ -119,7 +120,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
                  "fdfd_objective", "fdfd_grad", "fdfd_apply", "fdfd_set_options", "fdfd_stats_get",
                  "fdfd_plan_fronts", "fdfd_profile_enable", "fdfd_profile_get", "fdfd_filter_project",
                  "fdfd_filter_project_adjoint", "fdfd_objective_target", "fdfd_design_iteration",
-                 "fdfd_density_eps", "fdfd_front_copy", "fdfd_plan_sizes", "fdfd_selftest_mbar_wait", "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_sweep",
+                 "fdfd_density_eps", "fdfd_front_copy", "fdfd_plan_sizes", "fdfd_sweep_units", "fdfd_selftest_mbar_wait", "fdfd_selftest_wait", "fdfd_selftest_wait_async", "fdfd_selftest_sweep",
                  "fdfd_selftest_schur_tc", "fdfd_slab_modes"):
         getattr(lib, name).restype = C.c_int
     return lib
@@ -397,6 +398,12 @@ class Solver:
         iv = np.zeros((int(k[f]), max(1, int(ldk[f]))), dt)
         self._check(_lib.fdfd_front_copy(self._h, int(w), int(f), fr.ctypes.data, iv.ctypes.data), "fdfd_front_copy")
         return fr, iv
+
+    def sweep_units(self, sweep: int, f64: bool = False) -> dict:
+        """Work units of a sweep (0 L, 1 U, 2 U^T, 3 L^T) by kind; *_parts: those with several parts."""
+        c = np.zeros(7, np.int32)
+        self._check(_lib.fdfd_sweep_units(self._h, int(f64), int(sweep), c.ctypes.data), "fdfd_sweep_units")
+        return dict(zip(("small", "packed", "front", "tri", "rect", "tri_parts", "rect_parts"), map(int, c)))
 
     def plan_fronts(self):
         """(k, m, parent, level, design, idx) of the symbolic plan as numpy arrays."""
