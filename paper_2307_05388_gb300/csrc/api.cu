@@ -114,8 +114,8 @@ struct fdfd_ctx {
   SweepFront* d_sweepf = nullptr;  // the fronts as the sweeps read them, by level
   std::vector<SweepFront> h_sweepf;
   unsigned char* d_meta = nullptr; // index data of the packed fronts
-  std::vector<unsigned char> h_meta;
-  std::vector<size_t> h_moff;      // where record i's index data starts
+  size_t* d_moff = nullptr;        // where record i's index data starts
+  std::vector<size_t> h_moff;
   std::vector<int> h_first;        // records of level l: [h_first[l], h_first[l + 1])
   SweepUnit* d_units[2] = {nullptr, nullptr};
   std::vector<SweepUnit> h_units[2];
@@ -265,8 +265,8 @@ struct Prof {
 void free_plan_device(fdfd_ctx* c) {
   free_ptr(c->d_fronts); free_ptr(c->d_children); free_ptr(c->d_idx); free_ptr(c->d_inv);
   free_ptr(c->d_orig_ptr); free_ptr(c->d_orig_col); free_ptr(c->d_orig_code); free_ptr(c->d_lists);
-  free_ptr(c->d_sweepf); free_ptr(c->d_meta);
-  c->d_sweepf = nullptr; c->d_meta = nullptr;
+  free_ptr(c->d_sweepf); free_ptr(c->d_meta); free_ptr(c->d_moff);
+  c->d_sweepf = nullptr; c->d_meta = nullptr; c->d_moff = nullptr;
   for (int i = 0; i < 2; ++i) {
     free_ptr(c->d_units[i]); free_ptr(c->d_need[i]);
     c->d_units[i] = nullptr; c->d_need[i] = nullptr;
@@ -358,22 +358,18 @@ constexpr int kFlowCtasNarrow = 1;
 
 long long round16(long long b) { return (b + 15) / 16 * 16; }
 
-// The sweeps' records of the fronts and the packed fronts' index data (sweep.h), in sweep order.
+// The sweeps' records of the fronts, in sweep order, and where the packed fronts' index data (sweep.h, written by
+// launch_meta) goes.
 void build_records(fdfd_ctx* ctx) {
   const Plan& p = ctx->plan;
   const size_t nf = p.fronts.size();
   std::vector<SweepFront>& recs = ctx->h_sweepf;
-  std::vector<unsigned char>& meta = ctx->h_meta;
   std::vector<size_t>& moff = ctx->h_moff;
   std::vector<int>& first = ctx->h_first;
   recs.clear();
   recs.reserve(nf);
   moff.assign(nf + 1, 0);
   first.assign(p.n_levels + 1, 0);
-  size_t bytes = 0;
-  for (const FrontDesc& d : p.fronts)
-    if (d.n <= kPackMaxN) bytes += meta_bytes(d.n);
-  meta.assign(bytes, 0);
   ctx->ent_lower = ctx->ent_upper = ctx->ent_rect = 0;
   for (int f : p.sweep_order) {
     const FrontDesc& d = p.fronts[f];
@@ -394,17 +390,7 @@ void build_records(fdfd_ctx* ctx) {
     const size_t i = recs.size();
     recs.push_back(r);
     first[d.level + 1] = (int)i + 1;
-    moff[i + 1] = moff[i];
-    if (d.n <= kPackMaxN) {
-      unsigned char* o = meta.data() + moff[i];
-      std::memcpy(o, &r, sizeof(r));
-      std::memcpy(o + 96, &p.idx[d.idx_off], sizeof(int) * d.n);
-      unsigned* s = reinterpret_cast<unsigned*>(o + 96 + sizeof(int) * d.n);
-      for (int t = 0; t < d.n; ++t)
-        s[t] = (r.inv0 >= 0 ? (unsigned)p.inv[r.inv0 + t] & 0xffffu : 0xffffu) |
-               (r.inv1 >= 0 ? (unsigned)p.inv[r.inv1 + t] & 0xffffu : 0xffffu) << 16;
-      moff[i + 1] += meta_bytes(d.n);
-    }
+    moff[i + 1] = moff[i] + (d.n <= kPackMaxN ? meta_bytes(d.n) : 0);
     ctx->ent_lower += 0.5 * d.k * (d.k - 1.0);
     ctx->ent_upper += 0.5 * d.k * (d.k + 1.0);
     ctx->ent_rect += (double)d.k * d.m;
@@ -767,7 +753,9 @@ fdfd_status upload_plan(fdfd_ctx* ctx) {
   ctx->h_lists.swap(lists);
   CKS(upload(ctx, &ctx->d_lists, ctx->h_lists));
   CKS(upload(ctx, &ctx->d_sweepf, ctx->h_sweepf));
-  CKS(upload(ctx, &ctx->d_meta, ctx->h_meta));
+  CKS(upload(ctx, &ctx->d_moff, ctx->h_moff));
+  CK(dalloc(&ctx->d_meta, ctx->h_moff.back()));
+  CK(launch_meta(ctx->d_sweepf, (int)p.fronts.size(), ctx->d_moff, ctx->d_idx, ctx->d_inv, ctx->d_meta, ctx->stream));
   ctx->h_tcf.swap(tcf);
   ctx->h_tct.swap(tct);
   if (!ctx->h_tcf.empty()) {

@@ -198,6 +198,9 @@ constexpr int kFlowWideCtas = 2;      // per SM
 template <typename T> void launch_sweep_flow(const SolveLaunch& a, int sweep, const FlowQueue& q, const FlowShape& sh,
                                              int grid, const void* in, void* out, cudaStream_t s);
 int flow_blocks_per_sm(int elem_bytes, const FlowShape& sh);
+// index data of the packed fronts among the n records (sweep.h), each from moff[record] on
+cudaError_t launch_meta(const SweepFront* fronts, int n, const size_t* moff, const int* idx, const int* inv,
+                        unsigned char* meta, cudaStream_t s);
 // one bounded wait on a zero flag (gives up, sets *err); for the self-test entry point
 cudaError_t launch_wait_probe(const int* flag, int* err, cudaStream_t s);
 
