@@ -81,6 +81,7 @@ struct fdfd_ctx {
   std::vector<GraphEntry> graphs;
   std::string err;
   int device = -1;
+  int nsm = 1;                     // its SMs
 
   Plan plan;
   bool analyzed = false;
@@ -465,7 +466,7 @@ void build_units(fdfd_ctx* ctx, int prec) {
   units.clear();
   need_lists.assign((size_t)8 * nf, 0);                  // per sweep: all units of each front, its phase-1 units
   for (int sweep = 0; sweep < 4; ++sweep) {
-    const bool up = sweep == 0 || sweep == 2, rows = sweep < 2;
+    const bool up = sweep == 0 || sweep == 2;
     auto& fl = ctx->flow[prec][sweep];
     fl.uoff = units.size();
     int* all = need_lists.data() + (size_t)(2 * sweep) * nf;
@@ -777,6 +778,7 @@ fdfd_status ensure_runtime(fdfd_ctx* ctx) {
   if (ctx->device < 0) {
     int dev = -1;
     CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, dev));
     CK(factor_init_attributes());
     CK(panel_init_attributes());
     CK(tc_init_attributes());
@@ -960,8 +962,10 @@ fdfd_status factor_levels(fdfd_ctx* ctx, bool design_only, int w0 = 0, int nw = 
         {
           // block LU and inverses, L columns and U rows of the step (LU form: with the panel's update)
           Prof pr(ctx, PK_LU_STEP, (pf + lf + tf + (sym ? 0 : gf)) * nwd, (pb + lb + tb + (sym ? 0 : gb)) * nwd);
-          if (sym) launch_lu_step_local<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
-          else launch_panel_step<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
+          if constexpr (sizeof(T) == 8) {
+            if (sym) launch_lu_step_local<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
+          }
+          if (!sym) launch_panel_step<T>(fa, fl, ll.nlarge, j0, ll.nmax_large, s);
         }
         // block row J of L11^-1 and block column J of U11^-1: products with the
         // inverse so far, then with the block's own inverse
@@ -1296,7 +1300,7 @@ fdfd_status precond(fdfd_ctx* ctx, int nrhs, int transpose, const double2* src, 
 // split into more chunks).
 long long max_partials(const fdfd_ctx* ctx, int nrhs) {
   long long most = 1;
-  for (int r = 1; r <= nrhs; ++r) most = std::max(most, arnoldi_partials(n_cells(ctx), ctx->n_omega * r));
+  for (int r = 1; r <= nrhs; ++r) most = std::max(most, arnoldi_partials(n_cells(ctx), ctx->n_omega * r, ctx->nsm));
   return most;
 }
 
@@ -1406,7 +1410,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
   as.nj = ctx->d_nj; as.nj_out = ds.nj_out; as.active = ds.active; as.resid = ds.resid; as.bnorm = ctx->d_bnorm;
   as.vscale = ctx->d_vscale; as.H = ctx->d_H; as.cs = ctx->d_cs; as.sn = ctx->d_sn; as.g = ctx->d_g;
   as.loss = ctx->d_loss; as.reorth = ds.reorth; as.again = ctx->d_again; as.second = ctx->gm_second[tr] ? 1 : 0;
-  as.m = m; as.tol = tol; as.err = ctx->d_flow_err; as.err_out = ds.err;
+  as.m = m; as.nsm = ctx->nsm; as.tol = tol; as.err = ctx->d_flow_err; as.err_out = ds.err;
   { Prof pr(ctx, PK_DOT, 4.0 * N * S, 16.0 * N * S); launch_arnoldi(as, S, kPassStart, s); }
   CK(cudaGetLastError());
   long long total = 0;
@@ -1429,10 +1433,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
       if (wanted_second()) as.second = 1;
       if (!any) { converged = res <= tol; break; }   // a NaN residual is never converged
     }
-    if (total >= ctx->opt.ir_max_iter) {
-      if (cycle == 0) CK(cudaMemsetAsync(x, 0, sizeof(double2) * vs, s));
-      break;
-    }
+    if (total >= ctx->opt.ir_max_iter) break;      // (at least one: fdfd_solve sweeps without refinement at 0)
     { Prof pr(ctx, PK_OTHER, 0, 32.0 * N * S); gm_scale(ctx->d_V, cycle > 0 ? ctx->d_r : b, ctx->d_vscale, N, S, s); }
     int jdone = 0;
     for (int j = 0; j < m; ++j) {
@@ -1969,8 +1970,8 @@ fdfd_status fdfd_apply(fdfd_ctx* ctx, const double* x_dev, double* y_dev, int nr
   ctx->err.clear();
   if (!ctx->have_eps) return fail(ctx, FDFD_ERR_STATE, "fdfd_apply before fdfd_factor");
   CKS(ensure_runtime(ctx));
-  launch_stencil(dev_coef(ctx), ctx->n_omega, nrhs, transpose, reinterpret_cast<const double2*>(x_dev), nullptr,
-                 reinterpret_cast<double2*>(y_dev), 0, ctx->stream);
+  launch_stencil(dev_coef(ctx), ctx->n_omega, nrhs, transpose, reinterpret_cast<const double2*>(x_dev),
+                 reinterpret_cast<double2*>(y_dev), ctx->stream);
   CK(cudaGetLastError());
   return FDFD_OK;
 }

@@ -1198,9 +1198,7 @@ lu_step_local_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int 
   const int f = flist[blockIdx.y];
   const FrontDesc d = a.P.fronts[f];
   if (j0 >= d.k) return;
-  // L rows up to n; a front whose off-diagonal blocks come from the
-  // tensor cores stops at its pivot block
-  const int nb = min(kMaxNb, d.k - j0), n = (a.pivonly && a.pivonly[f]) ? d.k : d.n, ld = d.ld;
+  const int nb = min(kMaxNb, d.k - j0), n = d.n, ld = d.ld;
   const int bx = blockIdx.x + (phase == 2 ? 1 : 0);
   const size_t slot = (size_t)blockIdx.z * a.swp_stride + blockIdx.y;
   T* blk = reinterpret_cast<T*>(a.dblk) + slot * kDiagBlkElems;
@@ -1707,8 +1705,7 @@ lu_gemm_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nbmax,
   __shared__ T Bs[KC][kGemmTile + 1];
   __shared__ T dks[KC];                                 // symmetric form: d of the contracted pivots
   const int w = blockIdx.z + a.w0;
-  const int f = flist[blockIdx.y];
-  const FrontDesc d = a.P.fronts[f];
+  const FrontDesc d = a.P.fronts[flist[blockIdx.y]];
   if (!schur && j0 >= d.k) return;
   const int nb = schur ? d.k : min(nbmax, d.k - j0);   // contraction length
   const int kbeg = schur ? 0 : j0;                      // first contracted column of L / row of U
@@ -1720,9 +1717,6 @@ lu_gemm_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nbmax,
   const int ti = blockIdx.x / nt, tj = blockIdx.x - ti * nt;
   const int r0 = base + ti * kGemmTile, c0 = base + tj * kGemmTile;
   if (!schur && r0 >= d.k && c0 >= d.k) return;        // tile inside S: deferred to the Schur product
-  // a front whose off-diagonal blocks come from the tensor cores: the pivot block only
-  const bool pivonly = !schur && a.pivonly && a.pivonly[f];
-  if (pivonly && (r0 >= d.k || c0 >= d.k)) return;
   // symmetric form: the lower triangle only, and in a panel step only the pivot columns
   const bool sym = a.sym != 0;
   if (sym && (r0 + kGemmTile - 1 < c0 || (!schur && c0 >= d.k))) return;
@@ -1783,9 +1777,7 @@ lu_gemm_kernel(FactorLaunch a, const int* __restrict__ flist, int j0, int nbmax,
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int gc = c0 + tx + 16 * j;
-      const bool live = sym       ? (gr >= gc && (schur || gc < d.k))
-                        : pivonly ? (gr < d.k && gc < d.k)
-                                  : (schur || gr < d.k || gc < d.k);
+      const bool live = sym ? (gr >= gc && (schur || gc < d.k)) : (schur || gr < d.k || gc < d.k);
       if (gc < d.n && live) {
         T* p = F + (size_t)gr * d.ld + gc;
         *p = csub(*p, acc[i][j]);
@@ -1833,9 +1825,6 @@ cudaError_t factor_init_attributes() {
   e = cudaFuncSetAttribute(lu_step_local_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)step_local_smem(8));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(lu_step_local_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)step_local_smem(16));
-  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(lu_panel_smem_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kPanelSmemBytes);
   if (e != cudaSuccess) return e;
@@ -1847,8 +1836,12 @@ int lu_panel_width(int elem_bytes) { (void)elem_bytes; return kMaxNb; }
 template <typename T>
 void launch_build(const FactorLaunch& a, const int2* tasks, int ntasks, cudaStream_t s) {
   if (ntasks <= 0) return;
-  if (a.sym) build_kernel<T, true><<<dim3(ntasks, a.n_omega), kBuildWarps * 32, 0, s>>>(a, tasks);
-  else build_kernel<T, false><<<dim3(ntasks, a.n_omega), kBuildWarps * 32, 0, s>>>(a, tasks);
+  if constexpr (sizeof(T) == 8)
+    if (a.sym) {
+      build_kernel<T, true><<<dim3(ntasks, a.n_omega), kBuildWarps * 32, 0, s>>>(a, tasks);
+      return;
+    }
+  build_kernel<T, false><<<dim3(ntasks, a.n_omega), kBuildWarps * 32, 0, s>>>(a, tasks);
 }
 
 template <typename T>
@@ -1962,12 +1955,12 @@ void launch_lu_inv_fold(const FactorLaunch& a, const int* flist, int nf, int j0,
 template <typename T>
 void launch_schur_simt(const FactorLaunch& a, const int* flist, int nf, int mmax, cudaStream_t s) {
   if (nf <= 0 || mmax <= 0) return;
-  if (sizeof(T) == 16 && !a.sym) {
+  if constexpr (sizeof(T) == 16) {
     launch_schur_fine(a, flist, nf, mmax, s);
-    return;
+  } else {
+    const int nt = (mmax + kGemmTile - 1) / kGemmTile;
+    lu_gemm_kernel<T><<<dim3(nt * nt, nf, a.n_omega), 256, 0, s>>>(a, flist, 0, 0, 1);
   }
-  const int nt = (mmax + kGemmTile - 1) / kGemmTile;
-  lu_gemm_kernel<T><<<dim3(nt * nt, nf, a.n_omega), 256, 0, s>>>(a, flist, 0, 0, 1);
 }
 
 #define FDFD_INST(T)                                                                              \
@@ -1975,7 +1968,6 @@ void launch_schur_simt(const FactorLaunch& a, const int* flist, int nf, int mmax
   template void launch_lu_small<T>(const FactorLaunch&, const int*, int, int, cudaStream_t);      \
   template void launch_lu_panel<T>(const FactorLaunch&, const int*, int, int, int, int, cudaStream_t); \
   template void launch_lu_l21<T>(const FactorLaunch&, const int*, int, int, int, int, int, int, cudaStream_t); \
-  template void launch_lu_step_local<T>(const FactorLaunch&, const int*, int, int, int, cudaStream_t); \
   template void launch_lu_inv<T>(const FactorLaunch&, const int*, int, int, cudaStream_t); \
   template void launch_lu_trsm<T>(const FactorLaunch&, const int*, int, int, int, int, cudaStream_t); \
   template void launch_lu_gemm<T>(const FactorLaunch&, const int*, int, int, int, int, cudaStream_t); \
@@ -1984,5 +1976,6 @@ void launch_schur_simt(const FactorLaunch& a, const int* flist, int nf, int mmax
 FDFD_INST(float2)
 FDFD_INST(double2)
 #undef FDFD_INST
+template void launch_lu_step_local<float2>(const FactorLaunch&, const int*, int, int, int, cudaStream_t);
 
 }  // namespace fdfd

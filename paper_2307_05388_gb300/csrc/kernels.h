@@ -67,7 +67,7 @@ template <typename T> void launch_panel_step(const FactorLaunch& a, const int* f
 cudaError_t panel_init_attributes();
 // complex128, LU form: S = F22 - L21 U12 of the listed fronts (mmax = largest m listed)
 void launch_schur_fine(const FactorLaunch& a, const int* flist, int nf, int mmax, cudaStream_t s);
-// Symmetric form (no pivoting; L columns only): launch_lu_gemm does the trailing update.
+// Symmetric form (complex64; no pivoting, L columns only): launch_lu_gemm does the trailing update.
 template <typename T> void launch_lu_step_local(const FactorLaunch& a, const int* flist, int nf, int j0,
                                                 int nmax, cudaStream_t s);
 constexpr int kSwapScratchInts = 130;   // ints of swap scratch per (wavelength, listed front)
@@ -205,9 +205,9 @@ cudaError_t launch_meta(const SweepFront* fronts, int n, const size_t* moff, con
 cudaError_t launch_wait_probe(const int* flag, int* err, cudaStream_t s);
 
 // ---- vec.cu: FP64 refinement, objective, gradient ---------------------------
-// y = A x (op = 0) or r = b - A x (op = 1), FP64 matrix-free stencil, all systems.
-void launch_stencil(const DevCoef& c, int n_omega, int nrhs, int transpose, const double2* x,
-                    const double2* b, double2* y, int op, cudaStream_t s);
+// y = A x (or A^T x), FP64 matrix-free stencil, all systems.
+void launch_stencil(const DevCoef& c, int n_omega, int nrhs, int transpose, const double2* x, double2* y,
+                    cudaStream_t s);
 // w[s] -= sum_i h[s][i] V_i[s], or with set w[s] = -sum_i h[s][i] V_i[s]
 void launch_multiaxpy(const double2* V, long long vstride, int nv, const double2* h, int h_ld,
                       double2* w, long long n, int nsys, int set, cudaStream_t s);
@@ -227,7 +227,7 @@ struct ArnoldiStep {
   long long vstride;
   int nv;                  // V_0 .. V_{nv-1}; the step is j = nv - 1
   double2* w;              // the pass's vector: r, or the next Krylov vector
-  double2* partial;        // [arnoldi_partials(n, nsys)]
+  double2* partial;        // [arnoldi_partials(n, nsys, nsm)]
   int* cnt;                // [nsys] zero, left zero
   double2 *h1, *h2;        // projections, [nsys][multidot_max_vectors()]
   double2 *e2, *hn;        // squared norms (x) before and after a projection, [nsys]
@@ -243,12 +243,13 @@ struct ArnoldiStep {
   int* again;              // 1: kPassProj left the column to the second projection, [nsys]
   int second;              // the second projection's passes are launched
   int m;
+  int nsm;                 // SMs of the device
   double tol;
   const int* err;          // the sweeps' error word, copied beside the results by the passes that start a cycle
   int* err_out;
 };
 void launch_arnoldi(const ArnoldiStep& g, int nsys, int pass, cudaStream_t s);
-long long arnoldi_partials(long long n, int nsys);
+long long arnoldi_partials(long long n, int nsys, int nsm);
 
 // objective o = g^T x on a monitor column, F = sum weight |o|^2 with adjoint source weight conj(o) g,
 // or with target != NULL F = sum weight (|o|^2 - target)^2 with adjoint source 2 weight (|o|^2 - target) conj(o) g

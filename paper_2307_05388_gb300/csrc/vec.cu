@@ -95,19 +95,14 @@ __device__ __forceinline__ double2 stencil_at(const DevCoef& c, int w, int trans
   return acc;
 }
 
-// y = A x (op 0) or y = b - A x (op 1); transpose selects A^T.
+// y = A x; transpose selects A^T.
 __global__ void stencil_kernel(DevCoef c, int nrhs, int transpose, const double2* __restrict__ x,
-                               const double2* __restrict__ b, double2* __restrict__ y, int op) {
+                               double2* __restrict__ y) {
   const int sys = blockIdx.y;
   const long long N = (long long)c.nx * c.ny;
   const long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= N) return;
-  double2 acc = stencil_at(c, sys / nrhs, transpose, x + (size_t)sys * N, cell);
-  if (op == 1) {
-    const double2 bb = b[(size_t)sys * N + cell];
-    acc = make_double2(bb.x - acc.x, bb.y - acc.y);
-  }
-  y[(size_t)sys * N + cell] = acc;
+  y[(size_t)sys * N + cell] = stencil_at(c, sys / nrhs, transpose, x + (size_t)sys * N, cell);
 }
 
 constexpr int kDotThreads = 256;
@@ -149,10 +144,10 @@ void launch_scatter_design(double* eps, const double* eps_design, int ny, int x0
   scatter_design_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(eps, eps_design, ny, x0, y0, w, h);
 }
 
-void launch_stencil(const DevCoef& c, int n_omega, int nrhs, int transpose, const double2* x,
-                    const double2* b, double2* y, int op, cudaStream_t s) {
+void launch_stencil(const DevCoef& c, int n_omega, int nrhs, int transpose, const double2* x, double2* y,
+                    cudaStream_t s) {
   const long long N = (long long)c.nx * c.ny;
-  stencil_kernel<<<dim3((unsigned)((N + 255) / 256), n_omega * nrhs), 256, 0, s>>>(c, nrhs, transpose, x, b, y, op);
+  stencil_kernel<<<dim3((unsigned)((N + 255) / 256), n_omega * nrhs), 256, 0, s>>>(c, nrhs, transpose, x, y);
 }
 
 
@@ -465,18 +460,18 @@ void gm_scale(double2* dst, const double2* src, const double* scale, long long n
   scale_vec_kernel<<<dim3(grid_for(n), nsys), 256, 0, s>>>(dst, src, scale, n);
 }
 // Entries per thread: eight, but few enough that the CTAs still cover the SMs three times over.
-static int arnoldi_per(long long n, int nsys) {
+static int arnoldi_per(long long n, int nsys, int nsm) {
   int per = 8;
-  while (per > 1 && (n + kDotThreads * per - 1) / (kDotThreads * per) * nsys < 3 * 152) per /= 2;
+  while (per > 1 && (n + kDotThreads * per - 1) / (kDotThreads * per) * nsys < 3LL * nsm) per /= 2;
   return per;
 }
-long long arnoldi_partials(long long n, int nsys) {
-  const int per = arnoldi_per(n, nsys);
+long long arnoldi_partials(long long n, int nsys, int nsm) {
+  const int per = arnoldi_per(n, nsys, nsm);
   return (long long)nsys * (kMaxDot + 1) * ((n + kDotThreads * per - 1) / (kDotThreads * per));
 }
 void launch_arnoldi(const ArnoldiStep& g, int nsys, int pass, cudaStream_t s) {
   const long long n = (long long)g.C.nx * g.C.ny;
-  const int per = arnoldi_per(n, nsys);
+  const int per = arnoldi_per(n, nsys, g.nsm);
   const dim3 grid((unsigned)((n + kDotThreads * per - 1) / (kDotThreads * per)), nsys);
   switch (per) {
     case 8: arnoldi_kernel<8><<<grid, kDotThreads, 0, s>>>(g, pass); break;
