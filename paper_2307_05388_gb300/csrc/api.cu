@@ -1389,6 +1389,10 @@ fdfd_status any_active(fdfd_ctx* ctx, int S, bool inside, bool* any, double* max
 // Whether solves need the second projection is learnt from solves on the same preconditioner.
 void forget_second(fdfd_ctx* ctx) { ctx->gm_second[0] = ctx->gm_second[1] = false; }
 
+// Flops of a pass that applies A, per cell: the stencil between the absorbing layers (9 FP64 operations, three of
+// them multiply-adds), the difference from b or v_j and the squared norm.
+constexpr double kApplyFlops = 12 + 2 + 4;
+
 // Flexible GMRES, right-preconditioned by the cached LU, FP64 residuals and updates.
 fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int transpose) {
   const int m = std::max(1, std::min(ctx->opt.gmres_restart, multidot_max_vectors() - 1));
@@ -1421,7 +1425,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
     cycles = cycle;
     if (cycle > 0) {
       as.z = x; as.nv = 0; as.w = ctx->d_r;
-      Prof pr(ctx, PK_STENCIL, 52.0 * N * S, 56.0 * N * S);
+      Prof pr(ctx, PK_STENCIL, kApplyFlops * N * S, 56.0 * N * S);
       launch_arnoldi(as, S, kPassResid, s);
     }
     CK(cudaGetLastError());
@@ -1443,7 +1447,7 @@ fdfd_status fgmres(fdfd_ctx* ctx, const double2* b, double2* x, int nrhs, int tr
       // e = A z_j - v_j, its projection, |e|, Givens update
       as.z = Zj; as.nv = j + 1; as.w = ctx->d_w;
       const double pf = 8.0 * (j + 1) * N * S, pb = 16.0 * (j + 3) * N * S;
-      { Prof pr(ctx, PK_ARNOLDI, 54.0 * N * S + pf, 40.0 * N * S + 16.0 * (j + 1) * N * S);
+      { Prof pr(ctx, PK_ARNOLDI, kApplyFlops * N * S + pf, 40.0 * N * S + 16.0 * (j + 1) * N * S);
         launch_arnoldi(as, S, kPassApply, s); }
       { Prof pr(ctx, PK_ARNOLDI, pf + 4.0 * N * S, pb); launch_arnoldi(as, S, kPassProj, s); }
       if (as.second) {

@@ -51,3 +51,20 @@ def test_store_bytes_cover_the_factors(mode, es):
     k, m, *_ = (v.astype(float) for v in s.plan_fronts())
     assert s.stats()["store_bytes"] >= es * 3 * (2 * k * m + m * m).sum()
     s.close()
+
+
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_fgmres_flops_count_what_a_cell_takes(nrhs):
+    """Per cell: the operator between the absorbing layers, the difference and the norm 18, each projection or
+    update 8 a vector, the norm after it 4."""
+    wl, s = _solver()
+    b = torch.from_numpy(W.random_complex((2, nrhs, wl.n), 4)).cuda()
+    s.solve(b)
+    s.profile(True)
+    s.solve(b)
+    p, its = s.profile_get(), s.stats()["ir_iters"]
+    s.close()
+    assert p["stencil_f64"]["launches"] == 1 and p["gmres_arnoldi"]["launches"] == 2 * its      # one cycle
+    cells = 2 * nrhs * wl.n
+    assert p["stencil_f64"]["flops"] == 18 * cells
+    assert p["gmres_arnoldi"]["flops"] == sum(18 + 8 * j + 8 * j + 4 for j in range(1, its + 1)) * cells
