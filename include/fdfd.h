@@ -200,7 +200,9 @@ fdfd_status fdfd_refactor_design(fdfd_ctx* ctx, const double* eps_design_dev);
  * In mixed mode, refinement that stops above ir_tol on the complex FP32 factors
  * sends the factorisation to FP64 (counted in fdfd_stats.fallbacks) and the solve
  * is repeated; FDFD_ERR_NOT_CONVERGED (x holds the last iterate) is returned only
- * when it stops above ir_tol on FP64 factors as well. */
+ * when it stops above ir_tol on FP64 factors as well.  FDFD_ERR_STATE without a factorisation (plain
+ * mode makes its own).  A refined solve's digits below ir_tol can depend on the solves before it on
+ * the context, which size its first Krylov cycle; the same sequence of calls gives the same bits. */
 fdfd_status fdfd_solve(fdfd_ctx* ctx, const double* b_dev, double* x_dev, int nrhs, int transpose);
 
 /* Mode-overlap objective and its adjoint source (Eq. 4):

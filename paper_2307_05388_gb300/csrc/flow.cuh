@@ -38,7 +38,7 @@
 // Measured per launch, before (fronts' factor rows loaded by the warps that use
 // them, after the wait, one right-hand side after the other) and with this
 // scheme: 1760 x 1760, two wavelengths x two sources: L 3.37 -> 2.03 ms, U 2.60
-// -> 1.57, U^T 3.35 -> 2.16, L^T 2.82 -> 2.07 (a launch must read 3.4 GB of
+// -> 1.57, U^T 3.35 -> 2.16, L^T 2.82 -> 2.09 (a launch must read 3.4 GB of
 // factors, 0.5 ms); 100 x 100: 83 -> 43, 65 -> 44, 77 -> 45, 66 -> 51 us.  The
 // instructions of the small fronts' products and the gathers' latency bound it
 // now.  Not kept: four CTAs of four working warps per SM (L 2.41 ms), three of
